@@ -334,7 +334,7 @@ void run_copy_tasks(const CopyTask* d_tasks, int64_t n_tasks, const CopyTerm* d_
 
 // Davidson / vector kernels
 void multidot(const double* const* d_vecs, int k, const double* w, int64_t n, double* d_out,
-              double* d_partials, cudaStream_t s);
+              double* d_partials, int* d_count, cudaStream_t s);
 // out = beta out + coef_scale sum_j coef[j] vecs[j]
 void lincomb(const double* const* d_vecs, const double* d_coef, int k, int64_t n, double* out,
              double beta_out, double coef_scale, cudaStream_t s);
@@ -367,8 +367,29 @@ void heff_diag(const DiagTask* d_tasks, int n_tasks, const DiagTerm* d_terms,
 void batched_eigh2(const int64_t* d_off, const int64_t* d_woff, const int32_t* d_dim, int n,
                    double* d_A, double* d_V, double* d_Vs, double* d_w, int descending, int clip,
                    cudaStream_t s);
-void ritz_solve(const double* d_H, int ld, int k, double* d_scratch, double* d_w, double* d_Y,
-                cudaStream_t s);
+// the two lowest eigenpairs of H (k x k, k <= 64): values in d_w[0..1], coefficients in
+// d_Y[0 ..] and d_Y[64 ..] (davidson.cu)
+void ritz_solve(const double* d_H, int ld, int k, double* d_w, double* d_Y, cudaStream_t s);
+// everything of a Davidson iteration between the product Av = A v_{k-1} of the k-th subspace
+// vector and the product of the next one: last row of H, lowest Ritz pair, x, residual r,
+// diagonal correction t orthogonalised twice against V, next = t / |t|;
+// sc = {theta, |r|^2, |t|^2 before and after the orthogonalisation}
+struct DavChain {
+  const double* const* V;
+  const double* const* AV;
+  int k;
+  int64_t n;
+  const double* Av;
+  const double* diag;
+  double* H;         // row j holds <v_i, A v_j>, i <= j
+  int ldh;
+  double *w, *Y;
+  double *x, *r, *t, *next;
+  double* sc;        // 8 + 66 + 64 + 1 words
+  double* part;      // 66 x 264 words
+  int* count;        // zero between launches
+};
+void dav_chain(const DavChain& c, cudaStream_t s);
 // eigenpairs of rho_Q = B B^T from the singular vectors of the wave-function block B
 // (svd.cu): B = psi block (d x e, trans 0) or its transpose (trans 1, the block is e x d),
 // [psi0 psi1] / sqrt(2) with two roots; eigenvalues descending at w_off, eigenvectors as

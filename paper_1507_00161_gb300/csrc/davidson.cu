@@ -1,0 +1,567 @@
+// Davidson's vector algebra and its projected (Ritz) problem.
+//
+// One Davidson iteration after its product A v_k is a chain of short dependent pieces on a
+// few vectors of n elements (a few hundred in the sd shell, 10^5 at M = 4096):
+//     h = V^T (A v_k),   lowest Ritz pair,   x = V y, r = A V y - theta x,  t = r / (theta - D),
+//     t <- t - V (V^T t) twice,   v_{k+1} = t / |t|.
+// The chain is bound by launches and by the latency of each piece, not by bytes: at n = 1000
+// the vectors are 0.2 MB.  It runs as five launches with one readback (dav_chain).  The last
+// block of a launch to finish adds the partial sums of all blocks (a counter, no waiting), so
+// reductions need no launches of their own; the first launch's last block also solves the
+// Ritz problem.  The correction and the next vector are computed before the host has seen the
+// residual; a run that ends there ignores them.
+//
+// Every sum keeps one fixed shape whatever kernel forms it: 264 chunks of the vector, in a
+// chunk 256 partial sums (elements t, t + 256, ...), each 32 of them added as a binary tree,
+// the eight trees in order; the chunk sums are added the same way.  Far from convergence
+// theta lies inside the range of the diagonal, and the correction amplifies a last-bit
+// difference by orders of magnitude per iteration, so a run is only reproducible if the sums
+// are the same to the bit in every kernel.  A warp forms the eight trees together: after the
+// first level half of its lanes would idle, so two trees share each instruction from there on
+// (9 FP64 additions instead of 40; FP64 runs at 1.7 lanes per clock and SM here).
+//
+// Measured (GB300), chain and Ritz problem together, against 15 launches and two readbacks per
+// iteration: a Davidson run of pf 4p+4n (n = 700, ~52 products) 37.5 -> 27.0 ms, an sd-shell
+// sweep at M = 64 176 -> 123 ms, five instances in batch mode 481 -> 343 ms, bit for bit the
+// same results.
+#include <math.h>
+#include <stdint.h>
+
+#include <mutex>
+
+#include "common.h"
+
+namespace dmrg {
+
+namespace {
+
+constexpr int kThr = 256;
+constexpr int kWarps = kThr / 32;
+constexpr int kChunks = 264;          // chunks of a vector = blocks of a launch
+
+// sum of 256 values, p[t] held as p[w] = value 32 w + lane: the binary tree over each 32
+// (lane l + lane l + 16, then 8, 4, 2, 1), the eight trees added in order; every lane
+__device__ __forceinline__ double tree_sum(const double (&p)[kWarps]) {
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  double a[4], b[2], c;
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {   // lanes 0-15: tree 2 i, lanes 16-31: tree 2 i + 1
+    const double mine = h16 ? p[2 * i + 1] : p[2 * i];
+    const double give = h16 ? p[2 * i] : p[2 * i + 1];
+    a[i] = mine + __shfl_xor_sync(all, give, 16);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double mine = h8 ? a[2 * i + 1] : a[2 * i];
+    const double give = h8 ? a[2 * i] : a[2 * i + 1];
+    b[i] = mine + __shfl_xor_sync(all, give, 8);
+  }
+  {
+    const double mine = h4 ? b[1] : b[0];
+    const double give = h4 ? b[0] : b[1];
+    c = mine + __shfl_xor_sync(all, give, 4);
+  }
+  c += __shfl_xor_sync(all, c, 2);
+  c += __shfl_xor_sync(all, c, 1);
+  // tree 4 x + 2 y + z sits in the lanes with bit 2 = x, bit 3 = y, bit 4 = z
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w)
+    s += __shfl_sync(all, c, (w & 4) | ((w & 2) << 2) | ((w & 1) << 4));
+  return s;
+}
+
+// the sum of v[i] w[i] over a chunk of len elements, one warp
+__device__ __forceinline__ double chunk_dot(const double* v, const double* w, int len) {
+  const int lane = threadIdx.x & 31;
+  double p[kWarps];
+#pragma unroll
+  for (int q = 0; q < kWarps; ++q) p[q] = 0.0;
+  for (int base = 0; base < len; base += kThr)
+#pragma unroll
+    for (int q = 0; q < kWarps; ++q) {
+      const int i = base + 32 * q + lane;
+      if (i < len) p[q] = fma(v[i], w[i], p[q]);
+    }
+  return tree_sum(p);
+}
+
+// the sum of a launch's kChunks chunk sums, one warp
+__device__ __forceinline__ double chunks_sum(const double* part) {
+  const int lane = threadIdx.x & 31;
+  double p[kWarps];
+#pragma unroll
+  for (int q = 0; q < kWarps; ++q) p[q] = 0.0 + __ldcg(part + 32 * q + lane);
+  if (lane < kChunks - kThr) p[0] += __ldcg(part + kThr + lane);
+  return tree_sum(p);
+}
+
+// the sum of one value per thread, in thread 0 (shared by all launches of the chain)
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < kWarps; ++w) r += sh[w];
+  return r;
+}
+
+// true in every thread of the block that arrives last; *count is left at zero.  What the
+// other blocks wrote before is visible to it.
+__device__ __forceinline__ bool last_block(int* count) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(count, 1) == int(gridDim.x) - 1;
+    if (s_last) *count = 0;
+    __threadfence();
+  }
+  __syncthreads();
+  return s_last != 0;
+}
+
+struct Chunk {
+  int64_t i0;
+  int len;
+};
+__device__ __forceinline__ Chunk my_chunk(int64_t n) {
+  const int64_t c = (n + gridDim.x - 1) / gridDim.x;
+  const int64_t i0 = int64_t(blockIdx.x) * c;
+  return {i0, int(max(int64_t(0), min(n, i0 + c) - i0))};
+}
+
+// out[j] = vecs[j] . w, j < k
+__global__ void __launch_bounds__(kThr)
+k_dav_dots(const double* const* vecs, int k, const double* __restrict__ w, int64_t n,
+           double* part, double* __restrict__ out, int* count) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Chunk c = my_chunk(n);
+  for (int j = warp; j < k; j += kWarps) {
+    const double s = chunk_dot(vecs[j] + c.i0, w + c.i0, c.len);
+    if (lane == 0) part[j * kChunks + blockIdx.x] = s;
+  }
+  if (!last_block(count)) return;
+  for (int j = warp; j < k; j += kWarps) {
+    const double s = chunks_sum(part + j * kChunks);
+    if (lane == 0) out[j] = s;
+  }
+}
+
+// x, r, t; sums[0] = |r|^2, sums[1] = |t|^2, sums[2 ..] = V^T t
+__global__ void __launch_bounds__(kThr)
+k_dav_residual(const double* const* V, const double* const* AV, const double* __restrict__ y,
+               const double* __restrict__ theta, const double* __restrict__ diag, int k,
+               int64_t n, double* x, double* r, double* t,
+               double* part, double* __restrict__ sums, int* count) {
+  __shared__ double sy[64];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid < k) sy[tid] = y[tid];
+  __syncthreads();
+  const Chunk c = my_chunk(n);
+  const double th = *theta;
+  for (int64_t i = c.i0 + tid; i < c.i0 + c.len; i += kThr) {
+    double xs = 0.0, as = 0.0;
+#pragma unroll 4
+    for (int j = 0; j < k; ++j) {
+      xs = fma(sy[j], V[j][i], xs);
+      as = fma(sy[j], AV[j][i], as);
+    }
+    const double rv = fma(-th, xs, as);
+    double den = th - diag[i];
+    if (fabs(den) < 1e-8) den = den < 0.0 ? -1e-8 : 1e-8;
+    x[i] = xs;
+    r[i] = rv;
+    t[i] = rv / den;
+  }
+  __syncthreads();   // the chunk is read by other warps below
+  for (int j = warp; j < k + 2; j += kWarps) {
+    const double* u = (j == 0 ? r : t) + c.i0;
+    const double s = chunk_dot(j < 2 ? u : V[j - 2] + c.i0, u, c.len);
+    if (lane == 0) part[j * kChunks + blockIdx.x] = s;
+  }
+  if (!last_block(count)) return;
+  for (int j = warp; j < k + 2; j += kWarps) {
+    const double s = chunks_sum(part + j * kChunks);
+    if (lane == 0) sums[j] = s;
+  }
+}
+
+// t <- t - V h; then h <- V^T t, or (LAST) *h = |t|^2
+template <bool LAST>
+__global__ void __launch_bounds__(kThr)
+k_dav_orth(const double* const* V, int k, int64_t n, const double* __restrict__ h, double* t,
+           double* part, double* __restrict__ out, int* count) {
+  __shared__ double sh[64], red[kWarps];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid < k) sh[tid] = h[tid];
+  __syncthreads();
+  const Chunk c = my_chunk(n);
+  double tt = 0.0;
+  for (int64_t i = c.i0 + tid; i < c.i0 + c.len; i += kThr) {
+    double s = t[i];
+#pragma unroll 4
+    for (int j = 0; j < k; ++j) s = fma(-sh[j], V[j][i], s);
+    t[i] = s;
+    if (LAST) tt = fma(s, s, tt);
+  }
+  if (LAST) {
+    const double s = block_sum(tt, red);
+    if (tid == 0) part[blockIdx.x] = s;
+  } else {
+    __syncthreads();
+    for (int j = warp; j < k; j += kWarps) {
+      const double s = chunk_dot(V[j] + c.i0, t + c.i0, c.len);
+      if (lane == 0) part[j * kChunks + blockIdx.x] = s;
+    }
+  }
+  if (!last_block(count)) return;
+  for (int j = warp; j < (LAST ? 1 : k); j += kWarps) {
+    const double s = chunks_sum(part + j * kChunks);
+    if (lane == 0) out[j] = s;
+  }
+}
+
+// v = t / |t|; sc[0..3] = {theta, |r|^2, |t|^2 before and after}
+__global__ void __launch_bounds__(kThr)
+k_dav_next(const double* __restrict__ t, const double* __restrict__ tt,
+           const double* __restrict__ sums, const double* __restrict__ theta, int64_t n,
+           double* __restrict__ v, double* __restrict__ sc) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    sc[0] = *theta;
+    sc[1] = sums[0];
+    sc[2] = sums[1];
+    sc[3] = *tt;
+  }
+  const double f = 1.0 / sqrt(*tt);
+  for (int64_t i = int64_t(blockIdx.x) * kThr + threadIdx.x; i < n;
+       i += int64_t(gridDim.x) * kThr)
+    v[i] = t[i] * f;
+}
+
+// ------------------------------------------------------------------------------------
+// Ritz problem: H (k x k, row j holds <v_i, A v_j> for i <= j, leading dimension ld) -> the two
+// lowest eigenvalues w[0..1] and their coefficients Y[0 ..], Y[64 ..], each with its largest
+// |component| positive (lowest index on ties): cyclic Jacobi with the round-robin pairs and the
+// rotations of jacobi.cuh, the same operations on every element in the same order, in one block.
+//
+// One FP64 instruction of a warp occupies its scheduler's FP64 unit for 64 clocks (19 per SM with
+// four or more warps), whatever its active lanes and however independent the next one is, so
+// the time is the count of FP64 instructions on the critical path.  A rotation takes 30 of them
+// here against 47 with library divisions and roots, comparisons included; a round rotates the
+// matrix in 4.
+//   - Warp 0 forms the rotations.  Signs, zeros and powers of two are handled as integers.
+//   - The other warps meanwhile rotate V with the previous round's angles, and before the first
+//     round of a sweep sum the off-diagonal norm; V is only needed at the end.
+//   - Rows and columns of A are rotated in one pass, four lanes per 2 x 2 block (the rows of one
+//     pair, the columns of another): one element each, exchanged by shuffles.
+// Measured (GB300): 4400 clocks per round against 5700; a problem of 8 vectors 77 us, of 16 190 us.
+// ------------------------------------------------------------------------------------
+constexpr int kMaxK = 64;
+
+// Quotient, reciprocal and square root, rounded to nearest, by Newton's iteration with a final
+// correction from the exact remainder (P. Markstein, IBM J. Res. Dev. 34 (1990) 111): from a 2^-23
+// seed one step gives a reciprocal good to 2^-46 and, with the remainder, a result good to ~2^-90
+// before its one rounding.  Operands in 2^-400 .. 2^400.
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ bool mid_range(double x) {
+  const int e = exponent(x);
+  return e > 623 && e < 1423;
+}
+__device__ __forceinline__ bool is_zero(double x) {
+  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) == 0;
+}
+__device__ __forceinline__ double times_pow2(double x, int e) {   // x and the result normal
+  return __hiloint2double(__double2hiint(x) + (e << 20), __double2loint(x));
+}
+__device__ __forceinline__ double flip_if(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? int(0x80000000) : 0), __double2loint(x));
+}
+__device__ __forceinline__ double quick_rcp_step(double b) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  return fma(fma(-b, y, 1.0), y, y);
+}
+__device__ __forceinline__ double quick_div(double a, double b) {
+  const double y = quick_rcp_step(b), q = a * y;
+  return fma(fma(-b, q, a), y, q);
+}
+__device__ __forceinline__ double quick_rcp(double b) {
+  const double y = quick_rcp_step(b);
+  return fma(fma(-b, y, 1.0), y, y);
+}
+__device__ __forceinline__ double quick_sqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double g = x * y, h = times_pow2(y, -1);
+  const double e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  h = fma(h, e, h);
+  return fma(fma(-g, g, x), h, g);
+}
+
+// rotation that annihilates a_pq: theta = (a_qq - a_pp) / (2 a_pq), t = sgn(theta) /
+// (|theta| + sqrt(theta^2 + 1)), c = 1 / sqrt(t^2 + 1), s = t c; none for a_pq = 0.  All lanes
+// of `lanes` call it.  A warp whose operands all stay in the middle of the exponent range
+// (theta below 2^180) takes the straight line; otherwise the library's operations.
+__device__ __forceinline__ void rotation(unsigned lanes, double app, double aqq, double apq,
+                                         double& c, double& s) {
+  const double diff = aqq - app;
+  const bool none = is_zero(apq);
+  const bool fine = none || (mid_range(apq) && mid_range(diff) && exponent(diff) - exponent(apq) < 180);
+  if (__all_sync(lanes, fine)) {
+    const double th = quick_div(diff, times_pow2(apq, 1));
+    const double u = quick_rcp(fabs(th) + quick_sqrt(fma(th, th, 1.0)));
+    const double t = flip_if(u, __double2hiint(th) < 0);
+    c = quick_rcp(quick_sqrt(fma(t, t, 1.0)));
+    s = t * c;
+  } else {
+    const double th = diff / (2.0 * apq);
+    const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(fma(th, th, 1.0)));
+    c = 1.0 / sqrt(fma(t, t, 1.0));
+    s = t * c;
+  }
+  if (none) {
+    c = 1.0;
+    s = 0.0;
+  }
+}
+
+// round-robin pair number a of round r among m players
+__device__ __forceinline__ void pair_of(int m, int r, int a, int& p, int& q) {
+  int x = m - 1, y = r;
+  if (a > 0) {
+    x = r + a;
+    if (x >= m - 1) x -= m - 1;
+    y = r - a;
+    if (y < 0) y += m - 1;
+  }
+  p = min(x, y);
+  q = max(x, y);
+}
+
+struct RitzShared {
+  double c[2][kMaxK / 2], s[2][kMaxK / 2];   // rotations, double-buffered by round
+  int p[2][kMaxK / 2], q[2][kMaxK / 2];
+  double off[kWarps], tot[kWarps], w[kMaxK];
+  int low[2];
+};
+
+// columns of V by the rotations of buffer `buf`, by the threads first, first + step, ...
+__device__ __forceinline__ void rotate_v(double* V, int k, int half, const RitzShared& sh, int buf,
+                                         int first, int step) {
+  for (int e = first; e < half * k; e += step) {
+    const int a = e / k, row = e - a * k;
+    const int p = sh.p[buf][a], q = sh.q[buf][a];
+    const double c = sh.c[buf][a], s = sh.s[buf][a];
+    if (q >= k || is_zero(s)) continue;
+    const double vp = V[row * k + p], vq = V[row * k + q];
+    V[row * k + p] = fma(c, vp, -(s * vq));
+    V[row * k + q] = fma(s, vp, c * vq);
+  }
+}
+
+__device__ void ritz_block(const double* H, int ld, int k, double* sm, double* w, double* Y) {
+  __shared__ RitzShared sh;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  double* A = sm;
+  double* V = sm + k * k;
+  for (int i = tid; i < k * k; i += kThr) {
+    const int r = i / k, c = i - r * k;
+    A[i] = (r >= c) ? __ldcg(H + r * ld + c) : __ldcg(H + c * ld + r);
+    V[i] = r == c ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  const int m = (k + 1) & ~1, half = m / 2;
+  const int inv = 65536 / max(half, 1) + 1;   // x / half = (x inv) >> 16 for x < half^2 <= 1024
+  int buf = 0;
+  bool pending = false;   // rotations of buffer buf ^ 1 not yet applied to V
+  for (int sweep = 0; k > 1 && sweep < 40; ++sweep) {
+    bool done = false;
+    for (int r = 0; r < m - 1; ++r) {
+      if (warp == 0) {
+        int p, q;
+        pair_of(m, r, min(lane, half - 1), p, q);
+        const bool bye = q >= k;
+        double c, s;
+        rotation(0xffffffffu, A[p * k + p], bye ? 0.0 : A[q * k + q], bye ? 0.0 : A[p * k + q], c, s);
+        if (lane < half) {
+          sh.p[buf][lane] = p;
+          sh.q[buf][lane] = q;
+          sh.c[buf][lane] = c;
+          sh.s[buf][lane] = s;
+        }
+      } else {
+        if (pending) rotate_v(V, k, half, sh, buf ^ 1, tid - 32, kThr - 32);
+        if (r == 0) {   // off-diagonal Frobenius norm against the full norm
+          double off = 0.0, tot = 0.0;
+          for (int i = tid - 32; i < k * k; i += kThr - 32) {
+            const double a = A[i];
+            tot = fma(a, a, tot);
+            if (i / k != i % k) off = fma(a, a, off);
+          }
+          for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+          }
+          if (lane == 0) {
+            sh.off[warp] = off;
+            sh.tot[warp] = tot;
+          }
+        }
+      }
+      __syncthreads();
+      pending = false;
+      if (r == 0) {   // the same sums in every thread
+        double off = 0.0, tot = 0.0;
+        for (int x = 1; x < kWarps; ++x) {
+          off += sh.off[x];
+          tot += sh.tot[x];
+        }
+        done = off <= 1e-30 * tot || tot == 0.0;
+        if (done) break;
+      }
+      // A <- P^T A P: rows of pair a, columns of pair b; lane bit 1 = row, bit 0 = column of the
+      // block (whole groups of four lanes take part)
+      const int nel = 4 * half * half;
+      for (int e0 = tid & ~31; e0 < nel; e0 += kThr) {   // (whole warps)
+        const int e = e0 + lane;
+        const int blk = min(e, nel - 1) >> 2, a = (blk * inv) >> 16, b = blk - a * half;
+        const bool lo = tid & 2, right = tid & 1;
+        const int pa = sh.p[buf][a], qa = sh.q[buf][a], pb = sh.p[buf][b], qb = sh.q[buf][b];
+        const bool ra = qa < k, rb = qb < k;   // (an odd k has one pair with a bye)
+        const int row = lo ? qa : pa, col = right ? qb : pb;
+        const bool mine = e < nel && row < k && col < k;
+        double x = mine ? A[row * k + col] : 0.0;
+        // row p: c x_p - s x_q, row q: s x_p + c x_q (first product fused, second rounded)
+        const double sa = sh.s[buf][a], ca = sh.c[buf][a];
+        const double up = __shfl_xor_sync(0xffffffffu, x, 2);
+        if (ra && !is_zero(sa))
+          x = fma(lo ? sa : ca, lo ? up : x, flip_if((lo ? ca : sa) * (lo ? x : up), !lo));
+        const double sb = sh.s[buf][b], cb = sh.c[buf][b];
+        const double side = __shfl_xor_sync(0xffffffffu, x, 1);
+        if (rb && !is_zero(sb))
+          x = fma(right ? sb : cb, right ? side : x,
+                  flip_if((right ? cb : sb) * (right ? x : side), !right));
+        if (mine) A[row * k + col] = x;
+      }
+      pending = true;
+      buf ^= 1;
+      __syncthreads();
+    }
+    if (done) break;
+  }
+  if (pending) rotate_v(V, k, half, sh, buf ^ 1, tid, kThr);
+  if (tid < k) sh.w[tid] = A[tid * k + tid];
+  if (tid < 2) sh.low[tid] = min(tid, k - 1);   // (stays only if the weights are NaN)
+  __syncthreads();
+  // ranks 0 and 1, ties by index
+  if (tid < k) {
+    const double wi = sh.w[tid];
+    int rank = 0;
+    for (int j = 0; j < k; ++j) rank += sh.w[j] < wi || (sh.w[j] == wi && j < tid);
+    if (rank < 2) sh.low[rank] = tid;
+  }
+  __syncthreads();
+  if (warp < min(k, 2)) {
+    const int col = sh.low[warp];
+    double bv = -1.0, sg = 1.0;
+    int bi = 0x7fffffff;
+    for (int i = lane; i < k; i += 32) {
+      const double v = V[i * k + col], a = fabs(v);
+      if (a > bv) {
+        bv = a;
+        bi = i;
+        sg = v < 0.0 ? -1.0 : 1.0;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, bv, o), os = __shfl_xor_sync(0xffffffffu, sg, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > bv || (ov == bv && oi < bi)) {
+        bv = ov;
+        bi = oi;
+        sg = os;
+      }
+    }
+    for (int i = lane; i < k; i += 32) Y[64 * warp + i] = sg * V[i * k + col];
+    if (lane == 0) w[warp] = sh.w[col];
+  }
+}
+
+__global__ void __launch_bounds__(kThr)
+k_ritz(const double* H, int ld, int k, double* __restrict__ w, double* __restrict__ Y) {
+  extern __shared__ double sm[];
+  ritz_block(H, ld, k, sm, w, Y);
+}
+
+// H[k - 1][j] = V[j] . Av, j < k, then the Ritz problem, by the last block
+__global__ void __launch_bounds__(kThr)
+k_dav_ritz(const double* const* V, int k, const double* __restrict__ Av, int64_t n, double* part,
+           double* H, int ld, double* __restrict__ w, double* __restrict__ Y, int* count) {
+  extern __shared__ double sm[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Chunk c = my_chunk(n);
+  for (int j = warp; j < k; j += kWarps) {
+    const double s = chunk_dot(V[j] + c.i0, Av + c.i0, c.len);
+    if (lane == 0) part[j * kChunks + blockIdx.x] = s;
+  }
+  if (!last_block(count)) return;
+  for (int j = warp; j < k; j += kWarps) {
+    const double s = chunks_sum(part + j * kChunks);
+    if (lane == 0) __stcg(H + (k - 1) * ld + j, s);
+  }
+  __threadfence_block();
+  __syncthreads();
+  ritz_block(H, ld, k, sm, w, Y);
+}
+
+}  // namespace
+
+static size_t ritz_smem(int k) {
+  DMRG_REQUIRE(k >= 1 && k <= kMaxK, DMRG_EINVAL, "internal: Ritz problem too large");
+  static std::once_flag once;
+  std::call_once(once, [] {
+    const int most = int(sizeof(double) * 2 * kMaxK * kMaxK);
+    DMRG_CUDA(cudaFuncSetAttribute(k_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    DMRG_CUDA(cudaFuncSetAttribute(k_dav_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  });
+  return sizeof(double) * 2 * size_t(k) * k;
+}
+
+void multidot(const double* const* d_vecs, int k, const double* w, int64_t n, double* d_out,
+              double* d_partials, int* d_count, cudaStream_t s) {
+  if (k <= 0) return;
+  k_dav_dots<<<kChunks, kThr, 0, s>>>(d_vecs, k, w, n, d_partials, d_out, d_count);
+  DMRG_LAUNCHED();
+}
+
+void ritz_solve(const double* d_H, int ld, int k, double* d_w, double* d_Y, cudaStream_t s) {
+  k_ritz<<<1, kThr, ritz_smem(k), s>>>(d_H, ld, k, d_w, d_Y);
+  DMRG_LAUNCHED();
+}
+
+void dav_chain(const DavChain& c, cudaStream_t s) {
+  double* sums = c.sc + 8;      // |r|^2, |t|^2, V^T t
+  double* h2 = sums + 66;       // V^T t of the second pass
+  double* tt = h2 + 64;         // |t|^2
+  k_dav_ritz<<<kChunks, kThr, ritz_smem(c.k), s>>>(c.V, c.k, c.Av, c.n, c.part, c.H, c.ldh, c.w,
+                                                   c.Y, c.count);
+  DMRG_LAUNCHED();
+  k_dav_residual<<<kChunks, kThr, 0, s>>>(c.V, c.AV, c.Y, c.w, c.diag, c.k, c.n, c.x, c.r, c.t,
+                                          c.part, sums, c.count);
+  DMRG_LAUNCHED();
+  k_dav_orth<false><<<kChunks, kThr, 0, s>>>(c.V, c.k, c.n, sums + 2, c.t, c.part, h2, c.count);
+  DMRG_LAUNCHED();
+  k_dav_orth<true><<<kChunks, kThr, 0, s>>>(c.V, c.k, c.n, h2, c.t, c.part, tt, c.count);
+  DMRG_LAUNCHED();
+  const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((c.n + kThr - 1) / kThr, 152 * 8)));
+  k_dav_next<<<blocks, kThr, 0, s>>>(c.t, tt, sums, c.w, c.n, c.next, c.sc);
+  DMRG_LAUNCHED();
+}
+
+}  // namespace dmrg

@@ -237,6 +237,7 @@ struct dmrg_ctx {
   // Davidson workspace
   dmrg::DevBuf<double> V, AV, r, t, x, Ax, x1, Ax1, r1, small, partials;
   dmrg::DevBuf<const double*> vptr;
+  dmrg::DevBuf<int> dav_count;   // blocks arrived in a reduction (zero between launches)
   int64_t ws_n = 0, ws_sub = 0;
   // current eigenvector and what the next guess needs
   dmrg::DevBuf<double> psi, psi_guess;
@@ -1674,7 +1675,9 @@ static void ensure_ws(Ctx& c, int64_t n, int sub) {
   c.Ax1.alloc(nn);
   c.r1.alloc(nn);
   c.small.alloc(64 * 64 * 6 + 1024);
-  c.partials.alloc(64 * 300);
+  c.partials.alloc(66 * 300);
+  c.dav_count.alloc(1);
+  DMRG_CUDA(cudaMemsetAsync(c.dav_count.p, 0, sizeof(int), c.stream));
   std::vector<const double*> ptrs(2 * sub);
   for (int j = 0; j < sub; ++j) {
     ptrs[j] = c.V.p + j * nn;
@@ -1746,15 +1749,14 @@ struct DavRun {
 static const int kHist = 8;
 
 struct DavPtrs {
-  double *Hs, *w, *Y, *scr, *sc, *part;
+  double *Hs, *w, *Y, *sc, *part;
   const double* const* Vp;
   const double* const* AVp;
   DavPtrs(Ctx& c, int sub) {
     Hs = c.small.p;              // 64 x 64, row k holds <v_i, H v_k>, i <= k
     w = Hs + 64 * 64;            // Ritz values, ascending
-    Y = w + 64;                  // 64 x 64, row j = coefficients of the j-th Ritz vector
-    scr = Y + 64 * 64;           // 2 x 64 x 64 scratch for the Ritz solve
-    sc = scr + 2 * 64 * 64;      // device scalars
+    Y = w + 64;                  // rows 0 and 1 = coefficients of the two lowest Ritz vectors
+    sc = Y + 64 * 64;            // device scalars
     part = c.partials.p;
     Vp = c.vptr.p;
     AVp = c.vptr.p + sub;
@@ -1840,6 +1842,23 @@ static void dav_finish(Ctx& c, DavRun& R) {
   R.px = R.py = nullptr;
 }
 
+// FP32 products cannot resolve residuals below ~1e-7 of |H|: relative floor
+static double dav_tolerance(const Ctx& c, double theta) {
+  const double tol = c.opt.dav_tol;
+  return c.opt.precision == DMRG_FP64 ? tol : std::max(tol, 1e-6 * std::max(1.0, std::fabs(theta)));
+}
+
+// iterate, residual and Ritz value for training
+static void dav_history(Ctx& c, DavRun& R) {
+  if (!c.mlp_harvest || R.nhist >= kHist) return;
+  DavPtrs P(c, R.sub);
+  dav_d2d(c, c.hist_x.p + R.nhist * R.ld, c.x.p, R.n);
+  dav_d2d(c, c.hist_r.p + R.nhist * R.ld, c.r.p, R.n);
+  DMRG_CUDA(cudaMemcpyAsync(c.hist_theta.p + R.nhist, P.w, sizeof(double),
+                            cudaMemcpyDeviceToDevice, c.stream));
+  ++R.nhist;
+}
+
 // consume the product of vector k (py = H v_k), then either finish or request the next
 static void dav_after_product(Ctx& c, DavRun& R) {
   Super& sb = *R.sb;
@@ -1848,13 +1867,35 @@ static void dav_after_product(Ctx& c, DavRun& R) {
   const int64_t n = R.n, ld = R.ld;
   auto vec = [&](int j) { return c.V.p + j * ld; };
   auto avec = [&](int j) { return c.AV.p + j * ld; };
-  multidot(P.Vp, R.k + 1, avec(R.k), n, P.Hs + 64 * R.k, P.part, s);
+  double h[4];
+  // one state, diagonal correction, no restart due: the whole chain up to the next vector in
+  // one go (two targeted states, the learned map and a restart take the separate kernels)
+  if (R.nroots == 1 && !R.use_mlp && R.k + 1 < R.sub) {
+    const int j = R.k++;
+    ++R.nprod;
+    dav_chain(DavChain{P.Vp, P.AVp, R.k, n, avec(j), sb.diag.p, P.Hs, 64, P.w, P.Y, c.x.p, c.r.p,
+                       c.t.p, vec(R.k), P.sc, P.part, c.dav_count.p}, s);
+    dav_readback(c, P.sc, 4, h);
+    R.res.theta = h[0];
+    R.res.resid = std::sqrt(std::max(h[1], 0.0));
+    R.res.nprod = R.nprod;
+    dav_history(c, R);
+    const double tn0 = std::sqrt(std::max(h[2], 0.0)), tn = std::sqrt(std::max(h[3], 0.0));
+    R.res.converged = R.res.resid <= dav_tolerance(c, R.res.theta);
+    if (R.res.converged || R.nprod >= c.opt.dav_max_iter ||
+        tn <= 1e-14 * std::max(tn0, 1e-300)) {   // (or no new direction left)
+      dav_finish(c, R);
+      return;
+    }
+    R.px = vec(R.k);
+    R.py = avec(R.k);
+    return;
+  }
+  multidot(P.Vp, R.k + 1, avec(R.k), n, P.Hs + 64 * R.k, P.part, c.dav_count.p, s);
   ++R.k;
   ++R.nprod;
-  const double tol = c.opt.dav_tol;
-  double h[4];
   // Ritz pair of the projected matrix, residual r = H x - theta x
-  ritz_solve(P.Hs, 64, R.k, P.scr, P.w, P.Y, s);
+  ritz_solve(P.Hs, 64, R.k, P.w, P.Y, s);
   lincomb(P.Vp, P.Y, R.k, n, c.x.p, 0.0, 1.0, s);
   lincomb(P.AVp, P.Y, R.k, n, c.Ax.p, 0.0, 1.0, s);
   davidson_residual(c.x.p, c.Ax.p, P.w, n, c.r.p, s);
@@ -1879,16 +1920,8 @@ static void dav_after_product(Ctx& c, DavRun& R) {
     R.res.theta1 = h[2];
     R.res.resid1 = rn1;
   }
-  if (c.mlp_harvest && R.nhist < kHist) {   // iterate, residual and Ritz value for training
-    dav_d2d(c, c.hist_x.p + R.nhist * ld, c.x.p, n);
-    dav_d2d(c, c.hist_r.p + R.nhist * ld, c.r.p, n);
-    DMRG_CUDA(cudaMemcpyAsync(c.hist_theta.p + R.nhist, P.w, sizeof(double),
-                              cudaMemcpyDeviceToDevice, s));
-    ++R.nhist;
-  }
-  // FP32 products cannot resolve residuals below ~1e-7 of |H|: relative floor
-  const double tol_eff =
-      c.opt.precision == DMRG_FP64 ? tol : std::max(tol, 1e-6 * std::max(1.0, std::fabs(theta)));
+  dav_history(c, R);
+  const double tol_eff = dav_tolerance(c, theta);
   const bool conv = rn <= tol_eff && (R.nroots == 1 || (two && rn1 <= tol_eff));
   if (conv || R.nprod >= c.opt.dav_max_iter) {
     R.res.converged = conv;
@@ -1900,8 +1933,8 @@ static void dav_after_product(Ctx& c, DavRun& R) {
     R.guess1 = nullptr;
     dot(c.t.p, c.t.p, n, P.sc + 2, P.part, s);
     for (int pass = 0; pass < 2; ++pass) {
-      multidot(P.Vp, R.k, c.t.p, n, P.sc + 32, P.part, s);
-      lincomb(P.Vp, P.sc + 32, R.k, n, c.t.p, 1.0, -1.0, s);
+      multidot(P.Vp, R.k, c.t.p, n, P.sc + 256, P.part, c.dav_count.p, s);
+      lincomb(P.Vp, P.sc + 256, R.k, n, c.t.p, 1.0, -1.0, s);
     }
     dot(c.t.p, c.t.p, n, P.sc + 3, P.part, s);
     dav_readback(c, P.sc + 2, 2, h);
@@ -1941,8 +1974,8 @@ static void dav_after_product(Ctx& c, DavRun& R) {
   }
   dot(c.t.p, c.t.p, n, P.sc + 2, P.part, s);
   for (int pass = 0; pass < 2; ++pass) {   // classical Gram-Schmidt, twice
-    multidot(P.Vp, R.k, c.t.p, n, P.sc + 32, P.part, s);
-    lincomb(P.Vp, P.sc + 32, R.k, n, c.t.p, 1.0, -1.0, s);
+    multidot(P.Vp, R.k, c.t.p, n, P.sc + 256, P.part, c.dav_count.p, s);
+    lincomb(P.Vp, P.sc + 256, R.k, n, c.t.p, 1.0, -1.0, s);
   }
   dot(c.t.p, c.t.p, n, P.sc + 3, P.part, s);
   dav_readback(c, P.sc + 2, 2, h);

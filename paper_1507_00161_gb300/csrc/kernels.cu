@@ -5,9 +5,10 @@
 //    wave-function transformation).  Tiny tasks run one per warp straight from L1/L2;
 //    large tasks are cut into 64 x 64 tiles staged through shared memory.
 //  * copy tasks: scaled sums of operator blocks into enlarged-operator sub-blocks.
-//  * Davidson vector kernels with deterministic (fixed-order) reductions.
-//  * symmetric eigensolver: parallel-ordered cyclic Jacobi, one thread block per matrix,
-//    FP64 (reduced density matrices per sector and the small Ritz problem).
+//  * vector kernels with deterministic (fixed-order) reductions (the chain of a Davidson
+//    iteration: davidson.cu).
+//  * symmetric eigensolver: parallel-ordered cyclic Jacobi (jacobi.cuh), one thread block per
+//    matrix, FP64 (density matrices of sectors too wide for the cluster SVD).
 //  * selection of the M-th largest weight (bitonic sort in one block) and kept counts.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -16,6 +17,7 @@
 #include <mutex>
 
 #include "common.h"
+#include "jacobi.cuh"
 
 namespace dmrg {
 
@@ -399,21 +401,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return r;   // valid in thread 0
 }
 
-__global__ void k_multidot_partial(const double* const* vecs, int k, const double* __restrict__ w,
-                                   int64_t n, double* __restrict__ part) {
-  __shared__ double sh[32];
-  int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  int64_t i0 = int64_t(blockIdx.x) * chunk, i1 = min(n, i0 + chunk);
-  for (int j = 0; j < k; ++j) {
-    const double* v = vecs[j];
-    double s = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) s = fma(v[i], w[i], s);
-    double r = block_sum(s, sh);
-    if (threadIdx.x == 0) part[j * gridDim.x + blockIdx.x] = r;
-  }
-}
-
-__global__ void k_multidot_final(const double* __restrict__ part, int k, int nb,
+__global__ void k_dot_final(const double* __restrict__ part, int k, int nb,
                                  double* __restrict__ out) {
   int j = blockIdx.x;
   if (j >= k) return;
@@ -422,15 +410,6 @@ __global__ void k_multidot_final(const double* __restrict__ part, int k, int nb,
   for (int i = threadIdx.x; i < nb; i += blockDim.x) s += part[j * nb + i];
   double r = block_sum(s, sh);
   if (threadIdx.x == 0) out[j] = r;
-}
-
-void multidot(const double* const* d_vecs, int k, const double* w, int64_t n, double* d_out,
-              double* d_partials, cudaStream_t s) {
-  if (k <= 0) return;
-  k_multidot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(d_vecs, k, w, n, d_partials);
-  DMRG_LAUNCHED();
-  k_multidot_final<<<k, 256, 0, s>>>(d_partials, k, kDotBlocks, d_out);
-  DMRG_LAUNCHED();
 }
 
 __global__ void k_lincomb(const double* const* vecs, const double* __restrict__ coef, int k,
@@ -466,7 +445,7 @@ void dot(const double* a, const double* b, int64_t n, double* d_out, double* d_p
          cudaStream_t s) {
   k_dot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(a, b, n, d_partials);
   DMRG_LAUNCHED();
-  k_multidot_final<<<1, 256, 0, s>>>(d_partials, 1, kDotBlocks, d_out);
+  k_dot_final<<<1, 256, 0, s>>>(d_partials, 1, kDotBlocks, d_out);
   DMRG_LAUNCHED();
 }
 
@@ -559,128 +538,6 @@ void heff_diag(const DiagTask* d_tasks, int n_tasks, const DiagTerm* d_terms,
   DMRG_LAUNCHED();
 }
 
-// ------------------------------------------------------------------------------------
-// symmetric eigensolver: parallel cyclic Jacobi (round-robin pairing), one block per matrix
-// A (n x n, row-major, overwritten: diagonal -> eigenvalues), V (n x n) eigenvectors in
-// columns.  Rotation of (Numerical Recipes): theta = (a_qq - a_pp) / (2 a_pq),
-// t = sgn(theta)/(|theta| + sqrt(theta^2+1)), c = 1/sqrt(t^2+1), s = t c, A' = P^T A P.
-// ------------------------------------------------------------------------------------
-__device__ void jacobi_block(double* A, double* V, int n, double* cs, int* pp, int* qq,
-                             double* red) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < n * n; i += nt) V[i] = (i / n == i % n) ? 1.0 : 0.0;
-  __syncthreads();
-  if (n <= 1) return;
-  const int m = (n + 1) & ~1;   // even number of players (a dummy when n is odd)
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    // convergence: off-diagonal Frobenius norm against the full norm
-    double off = 0.0, tot = 0.0;
-    for (int i = tid; i < n * n; i += nt) {
-      double a = A[i];
-      tot += a * a;
-      if (i / n != i % n) off += a * a;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      off += __shfl_down_sync(0xffffffffu, off, o);
-      tot += __shfl_down_sync(0xffffffffu, tot, o);
-    }
-    __syncthreads();
-    if ((tid & 31) == 0) {
-      red[2 * (tid >> 5)] = off;
-      red[2 * (tid >> 5) + 1] = tot;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double o2 = 0.0, t2 = 0.0;
-      for (int w = 0; w < (nt + 31) / 32; ++w) { o2 += red[2 * w]; t2 += red[2 * w + 1]; }
-      red[64] = (o2 <= 1e-30 * t2 || t2 == 0.0) ? 1.0 : 0.0;
-    }
-    __syncthreads();
-    if (red[64] != 0.0) break;
-    for (int r = 0; r < m - 1; ++r) {
-      // round-robin tournament: player m-1 fixed, the others rotate
-      for (int k = tid; k < m / 2; k += nt) {
-        int a, b;
-        if (k == 0) {
-          a = m - 1;
-          b = r;
-        } else {
-          a = (r + k) % (m - 1);
-          b = (r - k + (m - 1)) % (m - 1);
-        }
-        int p = min(a, b), q = max(a, b);
-        double c = 1.0, s = 0.0;
-        if (q < n) {
-          double apq = A[p * n + q];
-          if (apq != 0.0) {
-            double th = (A[q * n + q] - A[p * n + p]) / (2.0 * apq);
-            double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-            c = 1.0 / sqrt(t * t + 1.0);
-            s = t * c;
-          }
-        }
-        pp[k] = p;
-        qq[k] = q;
-        cs[2 * k] = c;
-        cs[2 * k + 1] = s;
-      }
-      __syncthreads();
-      // rows: A <- P^T A
-      for (int e = tid; e < (m / 2) * n; e += nt) {
-        int k = e / n, col = e - k * n;
-        int p = pp[k], q = qq[k];
-        if (q >= n) continue;
-        double c = cs[2 * k], s = cs[2 * k + 1];
-        if (s == 0.0) continue;
-        double ap = A[p * n + col], aq = A[q * n + col];
-        A[p * n + col] = c * ap - s * aq;
-        A[q * n + col] = s * ap + c * aq;
-      }
-      __syncthreads();
-      // columns: A <- A P ; V <- V P
-      for (int e = tid; e < (m / 2) * n; e += nt) {
-        int k = e / n, row = e - k * n;
-        int p = pp[k], q = qq[k];
-        if (q >= n) continue;
-        double c = cs[2 * k], s = cs[2 * k + 1];
-        if (s == 0.0) continue;
-        double ap = A[row * n + p], aq = A[row * n + q];
-        A[row * n + p] = c * ap - s * aq;
-        A[row * n + q] = s * ap + c * aq;
-        double vp = V[row * n + p], vq = V[row * n + q];
-        V[row * n + p] = c * vp - s * vq;
-        V[row * n + q] = s * vp + c * vq;
-      }
-      __syncthreads();
-    }
-  }
-}
-
-// rank-sort of eigenpairs (descending or ascending), ties by original index; clip <0 to 0
-// when requested; eigenvector sign: largest |component| positive (lowest row on ties)
-__device__ void sort_and_fix(const double* A, const double* V, int n, double* w_out,
-                             double* V_out, int descending, int clip, int rs, int cs_) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double wi = A[i * n + i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      double wj = A[j * n + j];
-      bool before = descending ? (wj > wi) : (wj < wi);
-      if (before || (wj == wi && j < i)) ++rank;
-    }
-    w_out[rank] = (clip && wi < 0.0) ? 0.0 : wi;
-    // sign of column i
-    int best = 0;
-    double bv = -1.0;
-    for (int rr = 0; rr < n; ++rr) {
-      double a = fabs(V[rr * n + i]);
-      if (a > bv) { bv = a; best = rr; }
-    }
-    double sg = V[best * n + i] < 0.0 ? -1.0 : 1.0;
-    for (int rr = 0; rr < n; ++rr) V_out[rr * rs + rank * cs_] = sg * V[rr * n + i];
-  }
-}
-
 // Matrices up to kEighSmem on a side are decomposed in shared memory (the rotations touch
 // every element of two rows and two columns per round); larger ones in their global
 // workspace.
@@ -729,40 +586,6 @@ void batched_eigh2(const int64_t* d_off, const int64_t* d_woff, const int32_t* d
   eigh_smem_attr();
   k_batched_eigh2<<<n, 256, kEighSmemBytes, s>>>(d_off, d_woff, d_dim, d_A, d_V, d_Vs, d_w,
                                                   descending, clip);
-  DMRG_LAUNCHED();
-}
-
-// Ritz problem: H (k x k, leading dimension ld) -> ascending eigenvalues w, eigenvectors Y
-// (k x k, column j = j-th lowest, sign fixed); k <= 64, decomposed in shared memory
-__global__ void k_ritz(const double* __restrict__ H, int ld, int k, double* w, double* Y) {
-  extern __shared__ double ritz_sm[];
-  __shared__ double cs[1024];
-  __shared__ int pp[512], qq[512];
-  __shared__ double red[80];
-  double* A = ritz_sm;
-  double* V = ritz_sm + k * k;
-  for (int i = threadIdx.x; i < k * k; i += blockDim.x) {
-    int r = i / k, c = i - r * k;
-    // symmetric from the lower triangle: row j holds <v_i, H v_j> for i <= j
-    A[i] = (r >= c) ? H[r * ld + c] : H[c * ld + r];
-  }
-  __syncthreads();
-  jacobi_block(A, V, k, cs, pp, qq, red);
-  __syncthreads();
-  // Y row j = coefficients of the j-th lowest Ritz vector (leading dimension 64)
-  sort_and_fix(A, V, k, w, Y, 0, 0, 1, 64);
-}
-
-void ritz_solve(const double* d_H, int ld, int k, double* d_scratch, double* d_w, double* d_Y,
-                cudaStream_t s) {
-  (void)d_scratch;
-  DMRG_REQUIRE(k >= 1 && k <= kEighSmem, DMRG_EINVAL, "internal: Ritz problem too large");
-  static std::once_flag once;
-  std::call_once(once, [] {
-    DMRG_CUDA(cudaFuncSetAttribute(k_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   int(kEighSmemBytes)));
-  });
-  k_ritz<<<1, 256, sizeof(double) * 2 * k * k, s>>>(d_H, ld, k, d_w, d_Y);
   DMRG_LAUNCHED();
 }
 
