@@ -464,14 +464,18 @@ struct HeffItem {
 struct HeffTile {
   int64_t yoff;
   int64_t poff;
+  int64_t qoff;               // FP64 tile kernel: four partial tiles (heff.cu)
   int32_t ld;                 // dRo of the output block
   int32_t r0, c0, m, n;
   int32_t i0, i1;             // items [i0, i1)
   int32_t inst;               // instance (batch mode), 0 for one context
 };
-// deterministic sum of the partial tiles of one output tile
+// deterministic sum of the partial tiles of one output tile: `groups` tiles at poff, or (FP64
+// tile kernel) four per group at qoff.  A list holds the small-block tiles first, then the
+// tile kernels' tiles of several groups, then those of one group (which only the FP64 kernel
+// leaves as partial tiles)
 struct HeffRed {
-  int64_t yoff, poff;
+  int64_t yoff, poff, qoff;
   int32_t ld, r0, c0, m, n, groups;
   int32_t inst, pad;
 };
@@ -504,9 +508,10 @@ void heff_tc(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
 template <class TO>
 void pad_psi(const double* x, TO* xp, const int64_t* src_off, const int64_t* dst_off,
              const int32_t* len, int nblocks, cudaStream_t s);
-template <class T>
-void heff_fused(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
-                const HeffRed* d_red, int64_t n_red, const HeffPtrs<T>& ptrs, cudaStream_t s);
+// FP64 tile kernel and its sums (n_plain: small-block entries of the n_red)
+void heff_fused64(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
+                  const HeffRed* d_red, int64_t n_plain, int64_t n_red,
+                  const HeffPtrs<double>& ptrs, cudaStream_t s);
 // psi into / out of the 16-byte aligned staging copies, with the vector pointers read from
 // device memory (*xp_ptr, *out_ptr) so that a captured graph can be replayed on new vectors
 template <class TO>

@@ -171,7 +171,10 @@ struct Super {
   DevBuf<HeffItem> fitems;
   DevBuf<HeffTile> ftiles, stiles;   // tile kernels (32 x 32 tiles); small-block kernel
   DevBuf<HeffRed> fred;
-  int64_t n_ftiles = 0, n_stiles = 0, n_fred = 0, p_elems = 0;
+  // sums of partial tiles: small-block tiles, tiles of several groups, of one group (FP64 only)
+  int64_t n_ftiles = 0, n_stiles = 0, n_fred[3] = {0, 0, 0}, p_elems = 0, q_elems = 0;
+  int64_t reds_mixed() const { return n_fred[0] + n_fred[1]; }
+  int64_t reds64() const { return n_fred[0] + n_fred[1] + n_fred[2]; }
   std::vector<HeffItem> h_items;
   std::vector<HeffTile> h_tiles, h_stiles;
   std::vector<HeffRed> h_red;
@@ -1071,8 +1074,10 @@ static void build_super(Ctx& c, int p) {
   // small output blocks (every dimension of the block and of its terms <= kSmallEdge) are
   // single tiles of the warp kernel with groups of at most Gs terms
   const int G = 64, Gs = 16;
-  std::vector<int64_t> i_beg(nb + 1, 0), t_beg(nb + 1, 0), s_beg(nb + 1, 0), r_beg(nb + 1, 0),
-      p_beg(nb + 1, 0);
+  std::vector<int64_t> i_beg(nb + 1, 0), t_beg(nb + 1, 0), s_beg(nb + 1, 0), p_beg(nb + 1, 0),
+      q_beg(nb + 1, 0), r_beg(nb, 0);
+  int64_t n_red[3] = {0, 0, 0};   // reductions by class: small, several groups, one group
+  std::vector<char> red_class(nb, 0);
   std::vector<char> small_bo(nb, 0), big_bo(nb, 0);
   for (int bo = 0; bo < nb; ++bo) {
     const int ni = int(by_out[bo].size());
@@ -1091,7 +1096,12 @@ static void build_super(Ctx& c, int p) {
     i_beg[bo + 1] = i_beg[bo] + ni;
     t_beg[bo + 1] = t_beg[bo] + (sm || big ? 0 : tiles * groups);
     s_beg[bo + 1] = s_beg[bo] + (sm ? groups : 0);
-    r_beg[bo + 1] = r_beg[bo] + (groups > 1 && !big ? tiles : 0);
+    if (!big && !(sm && groups == 1)) {
+      red_class[bo] = sm ? 0 : groups > 1 ? 1 : 2;
+      r_beg[bo] = n_red[int(red_class[bo])];
+      n_red[int(red_class[bo])] += tiles;
+    }
+    q_beg[bo + 1] = q_beg[bo] + (sm || big ? 0 : int64_t(4) * groups * sb->bdl[bo] * sb->bdr[bo]);
     p_beg[bo + 1] = p_beg[bo] + (groups > 1 && !big ? int64_t(groups) * sb->bdl[bo] * sb->bdr[bo] : 0);
   }
   DMRG_REQUIRE(i_beg[nb] < (int64_t(1) << 31), DMRG_EINVAL, "superblock has too many terms");
@@ -1101,7 +1111,11 @@ static void build_super(Ctx& c, int p) {
   };
   std::vector<HeffItem> fi(i_beg[nb]);
   std::vector<TileCost> ft(t_beg[nb]), fts(s_beg[nb]);
-  std::vector<HeffRed> fr(r_beg[nb]);
+  std::vector<HeffRed> fr(n_red[0] + n_red[1] + n_red[2]);
+  for (int bo = 0; bo < nb; ++bo) {
+    if (red_class[bo] > 0) r_beg[bo] += n_red[0];
+    if (red_class[bo] > 1) r_beg[bo] += n_red[1];
+  }
   std::vector<double> bo_flops(nb, 0.0), bo_bytes(nb, 0.0), bo_kflops(nb, 0.0);
   std::vector<int64_t> bo_toff(nb, 0);
   std::vector<std::array<double, 8>> bo_hist(nb);
@@ -1149,6 +1163,7 @@ static void build_super(Ctx& c, int p) {
       const int GG = sm ? Gs : G, edge = sm ? kSmallEdge : 32;
       const int groups = std::max(1, (i1 - i0 + GG - 1) / GG);
       int64_t tpos = sm ? s_beg[bo] : t_beg[bo], rpos = r_beg[bo], pelems = p_beg[bo];
+      int64_t qelems = p_beg[nb] + q_beg[bo];
       std::vector<TileCost>& dst = sm ? fts : ft;
       for (int r0 = 0; r0 < dLo; r0 += edge)
         for (int c0 = 0; c0 < dRo; c0 += edge) {
@@ -1161,10 +1176,11 @@ static void build_super(Ctx& c, int p) {
           t.n = std::min(edge, dRo - c0);
           t.inst = 0;
           const int64_t mn = int64_t(t.m) * t.n;
-          if (groups > 1) {
+          if (groups > 1 || !sm) {
             HeffRed rd;
             rd.yoff = t.yoff;
             rd.poff = pelems;
+            rd.qoff = sm ? 0 : qelems;
             rd.ld = t.ld;
             rd.r0 = r0;
             rd.c0 = c0;
@@ -1179,9 +1195,11 @@ static void build_super(Ctx& c, int p) {
             t.i0 = i0 + g * GG;
             t.i1 = std::min(i1, t.i0 + GG);
             t.poff = groups > 1 ? pelems + g * mn : -1;
+            t.qoff = sm ? 0 : qelems + 4 * g * mn;
             dst[tpos++] = TileCost{t, work * double(t.i1 - t.i0) / std::max(1, i1 - i0) * t.n + 1.0};
           }
           if (groups > 1) pelems += groups * mn;
+          if (!sm) qelems += 4 * groups * mn;
         }
     }
   });
@@ -1198,7 +1216,7 @@ static void build_super(Ctx& c, int p) {
   c.kernel_flops = 0;
   for (int bo = 0; bo < nb; ++bo) c.kernel_flops += bo_kflops[bo];
   const int64_t items = i_beg[nb];
-  const int64_t pelems = p_beg[nb];
+  const int64_t pelems = p_beg[nb], qend = p_beg[nb] + q_beg[nb];
   sb->t_elems = toff;
   sb->n_items = items;
   c.last_sizes[0] = int64_t(sb->L.blocks.size());
@@ -1221,7 +1239,8 @@ static void build_super(Ctx& c, int p) {
         const HeffTile& t = v[i].t;
         tl[i] = t;
         DMRG_REQUIRE(t.m >= 1 && t.n >= 1 && t.m <= edge && t.n <= edge &&
-                         t.yoff + int64_t(t.r0 + t.m - 1) * t.ld + t.c0 + t.n - 1 < sb->size,
+                         t.yoff + int64_t(t.r0 + t.m - 1) * t.ld + t.c0 + t.n - 1 < sb->size &&
+                         (edge != 32 || t.qoff + int64_t(4) * t.m * t.n <= qend),
                      DMRG_EINVAL, "internal: fused tile out of range");
         for (int j = t.i0; j < t.i1; ++j) {
           const HeffItem& h = fi[j];
@@ -1237,7 +1256,8 @@ static void build_super(Ctx& c, int p) {
     check(ft, tl, 32);
     check(fts, tls, kSmallEdge);
     for (const HeffRed& r : fr)
-      DMRG_REQUIRE(r.poff + int64_t(r.groups) * r.m * r.n <= pelems &&
+      DMRG_REQUIRE((r.groups == 1 || r.poff + int64_t(r.groups) * r.m * r.n <= pelems) &&
+                       r.qoff + (r.qoff ? int64_t(4) * r.groups * r.m * r.n : 0) <= qend &&
                        r.yoff + int64_t(r.r0 + r.m - 1) * r.ld + r.c0 + r.n - 1 < sb->size,
                    DMRG_EINVAL, "internal: partial tile out of range");
     sb->fitems.upload(fi, c.stream);
@@ -1255,8 +1275,9 @@ static void build_super(Ctx& c, int p) {
     for (size_t i = 0; i < fts.size(); ++i) sb->h_scost[i] = fts[i].cost;
     sb->n_ftiles = int64_t(sb->h_tiles.size());
     sb->n_stiles = int64_t(sb->h_stiles.size());
-    sb->n_fred = int64_t(sb->h_red.size());
+    std::copy(n_red, n_red + 3, sb->n_fred);
     sb->p_elems = pelems;
+    sb->q_elems = q_beg[nb];
   }
   {
     // grouped GEMM passes of the big output blocks, each term in its cheaper association:
@@ -1322,6 +1343,7 @@ static void build_super(Ctx& c, int p) {
         HeffRed r;
         r.yoff = sb->boff[bo];
         r.poff = poff2;
+        r.qoff = 0;
         r.ld = dRo;
         r.r0 = 0;
         r.c0 = 0;
@@ -1435,7 +1457,7 @@ static void ensure_two_stage(Ctx& c, Super& sb) {
 // (and before a graph capture, which may not allocate)
 static void heff_buffers(Ctx& c, Super& sb, int prec) {
   if (prec == 0) {
-    c.part64.alloc(std::max<int64_t>(sb.p_elems, 1));
+    c.part64.alloc(std::max<int64_t>(sb.p_elems + sb.q_elems, 1));
     c.xpad64.alloc(sb.pad_size);
     c.ygraph64.alloc(std::max<int64_t>(sb.size, 1));
     if (sb.n_big_blocks) {
@@ -1467,8 +1489,8 @@ static void heff_core(Ctx& c, Super& sb, int prec, double* y64, cudaStream_t st)
     ptr.Y[0] = y64;
     ptr.P[0] = c.part64.p;
     heff_small<double>(sb.stiles.p, sb.n_stiles, sb.fitems.p, ptr, st);
-    heff_fused<double>(sb.ftiles.p, sb.n_ftiles, sb.fitems.p, sb.fred.p, sb.n_fred, ptr,
-                       st);
+    heff_fused64(sb.ftiles.p, sb.n_ftiles, sb.fitems.p, sb.fred.p, sb.n_fred[0], sb.reds64(), ptr,
+                 st);
     if (sb.n_big_blocks) {
       Bases<double> bb{};
       bb.p[B_LOPS] = sb.L.data.p;
@@ -1492,7 +1514,7 @@ static void heff_core(Ctx& c, Super& sb, int prec, double* y64, cudaStream_t st)
     ptr.Y[0] = c.f32b.p;
     ptr.P[0] = c.part32.p;
     heff_small<float>(sb.stiles.p, sb.n_stiles, sb.fitems.p, ptr, st);
-    heff_tc(sb.ftiles.p, sb.n_ftiles, sb.fitems.p, sb.fred.p, sb.n_fred, ptr, st);
+    heff_tc(sb.ftiles.p, sb.n_ftiles, sb.fitems.p, sb.fred.p, sb.reds_mixed(), ptr, st);
     if (sb.n_big_blocks) {
       Bases<void> bb{};
       bb.p[B_LOPS] = sb.L.data32.p;
@@ -1821,7 +1843,7 @@ static void dav_finish(Ctx& c, DavRun& R) {
     }
     if (!c.h_words) DMRG_CUDA(cudaMallocHost(&c.h_words, sizeof(double) * 64));
     c.rq_part.alloc(64 * 300);
-    c.part64.alloc(std::max<int64_t>(sb.p_elems, 1));
+    c.part64.alloc(std::max<int64_t>(sb.p_elems + sb.q_elems, 1));
     c.xpad64.alloc(sb.pad_size);
     DMRG_CUDA(cudaEventRecord(c.rq_in, c.stream));   // the normalized vector is ready
     c.rq_sb = &sb;
@@ -3785,7 +3807,7 @@ struct dmrg_batch {
   dmrg::DevBuf<dmrg::HeffItem> items;
   dmrg::DevBuf<dmrg::HeffTile> tiles, stiles;
   dmrg::DevBuf<dmrg::HeffRed> red;
-  int64_t n_tiles = 0, n_stiles = 0, n_red = 0;
+  int64_t n_tiles = 0, n_stiles = 0, n_red[3] = {0, 0, 0};   // (reductions by class, see Super)
   // per-iteration tables: input and output vector pointers, active flags
   struct Tab {
     const double* in[dmrg::kMaxInst];
@@ -3824,7 +3846,7 @@ struct PoolScope {
 static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
   std::vector<HeffItem> fi;
   std::vector<std::pair<double, HeffTile>> ft, fts;
-  std::vector<HeffRed> fr;
+  std::vector<HeffRed> fr[3];
   for (int i : inst) {
     Super& sb = *B.ctx[i]->sb;
     const int base = int(fi.size());
@@ -3841,10 +3863,13 @@ static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
     };
     add(sb.h_tiles, sb.h_cost, ft);
     add(sb.h_stiles, sb.h_scost, fts);
-    for (HeffRed r : sb.h_red) {
-      r.inst = i;
-      fr.push_back(r);
-    }
+    size_t at = 0;
+    for (int k = 0; k < 3; ++k)
+      for (int64_t x = 0; x < sb.n_fred[k]; ++x) {
+        HeffRed r = sb.h_red[at++];
+        r.inst = i;
+        fr[k].push_back(r);
+      }
   }
   auto sorted = [](std::vector<std::pair<double, HeffTile>>& v) {
     std::stable_sort(v.begin(), v.end(),
@@ -3857,10 +3882,13 @@ static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
   B.items.upload(fi, B.bs);
   B.tiles.upload(tl, B.bs);
   B.stiles.upload(tls, B.bs);
-  B.red.upload(fr, B.bs);
+  for (int k = 0; k < 3; ++k) {
+    B.n_red[k] = int64_t(fr[k].size());
+    if (k) fr[0].insert(fr[0].end(), fr[k].begin(), fr[k].end());
+  }
+  B.red.upload(fr[0], B.bs);
   B.n_tiles = int64_t(tl.size());
   B.n_stiles = int64_t(tls.size());
-  B.n_red = int64_t(fr.size());
   DMRG_CUDA(cudaStreamSynchronize(B.bs));
 }
 
@@ -3883,7 +3911,8 @@ static void batch_issue(dmrg_batch& B, const std::vector<int>& inst) {
       ptr.P[i] = c.part64.p;
     }
     heff_small<double>(B.stiles.p, B.n_stiles, B.items.p, ptr, B.bs);
-    heff_fused<double>(B.tiles.p, B.n_tiles, B.items.p, B.red.p, B.n_red, ptr, B.bs);
+    heff_fused64(B.tiles.p, B.n_tiles, B.items.p, B.red.p, B.n_red[0],
+                 B.n_red[0] + B.n_red[1] + B.n_red[2], ptr, B.bs);
     for (int i : inst) {   // big output blocks: grouped GEMM passes per instance
       Ctx& c = *B.ctx[i];
       Super& sb = *c.sb;
@@ -3922,7 +3951,7 @@ static void batch_issue(dmrg_batch& B, const std::vector<int>& inst) {
       ptr.P[i] = c.part32.p;
     }
     heff_small<float>(B.stiles.p, B.n_stiles, B.items.p, ptr, B.bs);
-    heff_tc(B.tiles.p, B.n_tiles, B.items.p, B.red.p, B.n_red, ptr, B.bs);
+    heff_tc(B.tiles.p, B.n_tiles, B.items.p, B.red.p, B.n_red[0] + B.n_red[1], ptr, B.bs);
     for (int i : inst) {   // big output blocks: grouped GEMM passes per instance
       Ctx& c = *B.ctx[i];
       Super& sb = *c.sb;
@@ -3956,7 +3985,7 @@ static void batch_buffers(dmrg_batch& B, const std::vector<int>& inst) {
     PoolScope ps(&c.pool);
     Super& sb = *c.sb;
     if (B.precision == DMRG_FP64) {
-      c.part64.alloc(std::max<int64_t>(sb.p_elems, 1));
+      c.part64.alloc(std::max<int64_t>(sb.p_elems + sb.q_elems, 1));
       c.xpad64.alloc(sb.pad_size);
       c.ybat64.alloc(std::max<int64_t>(sb.size, 1));
       if (sb.n_big_blocks) {

@@ -1,288 +1,178 @@
-// Fused superblock product  psi'(b') = sum_k s_k L_k[Q_L' <- Q_L] psi(b) R_k[Q_R' <- Q_R]^T
-// (the two-site H_eff of the superblock "Xi_l (x) Lambda (x) Lambda (x) Xi_r").
+// FP64 superblock product  psi'(b') = sum_k s_k L_k[Q_L' <- Q_L] psi(b) R_k[Q_R' <- Q_R]^T
+// (the two-site H_eff of the superblock "Xi_l (x) Lambda (x) Lambda (x) Xi_r") for the output
+// blocks between the small-block kernel and the grouped passes.
 //
-// Work unit (one thread block, four warps): a group of at most 64 terms of one output
-// tile (at most 32 x 32 of a psi' block).  Each warp takes every fourth term of the group.
-// Operator blocks and psi blocks start on 16-byte boundaries, so a warp streams the three
-// blocks of a term (L rows of the tile, R rows of the tile, psi_in) into a shared-memory
-// ring with 16-byte cp.async copies, up to four terms ahead of the one it computes
-// (completion in commit-group order; no spin-waits).  Compute from shared memory with a
-// fixed lane map: lane = (column c, row group g), rows g, g+G, ... with G = 32 / n:
-//     X[i][c] = sum_r psi[i][r] R[c][r]        (X in shared memory)
-//     acc[i][c] += s sum_k L[i][k] X[k][c]     (acc in registers)
-// Terms whose inner dimensions exceed 32 go through a chunked path that reads global
-// memory directly.  The warps' partial tiles are added in a fixed order, and groups of one
-// tile are added in group order by k_heff_reduce: the result is deterministic.
+// FP64 on this chip is one warp instruction per 19 clocks and SM (64 per scheduler), whatever the
+// instruction's active lanes and however independent the next one is.  So the kernel is bound by
+// the count of FP64 warp instructions, i.e. by lanes left idle, and by having four warps ready;
+// operand traffic is cheap beside it (two operands per 19 clocks).  Hence
+//   - the elements of a term's intermediate, and of the output tile, are numbered through and
+//     dealt to the warps 32 at a time (a 25 x 25 tile fills 20 instructions instead of 25 rows
+//     of 25 lanes), with one element per thread in flight and the sums in shared memory;
+//   - psi and L are read where they are (a warp reads one to three rows, broadcast from the L1);
+//     only the R tile is staged, because its rows run across the lanes;
+//   - a work unit is one output tile (at most 32 x 32), one group of at most 64 terms and one of
+//     four slots: every fourth term of the group, in order.  25 KB of shared memory and four
+//     warps per unit put eight units on an SM, so one unit's loads and barriers are covered by
+//     the others, and a superblock with few tiles still fills the chip.
+// Per term: X = psi R^T (chunks of 32 rows of psi), then acc += L (s X); terms small enough use
+// the cheaper association of the tile ((L psi) first).  The four slots of a group are added in
+// order and the groups in order by k_heff_reduce: the result is deterministic, and the same bit
+// for bit as one thread block running the group with one warp per slot.
+// Measured (GB300) against one thread block per group (a row of lanes per tile row, wide terms
+// staged in synchronous chunks): pf 8p+8n at position 12, M0 = 3000 (2.0 GFLOP) 9.48 -> 2.55 ms,
+// 0.78 of the 1.07 TFLOP/s that FP64 reaches here; pf 4p+4n at M = 1024, position 20 (0.25 GFLOP)
+// 1.99 -> 0.39 ms; pf 4p+4n, position 9, M0 = 256 (152 tiles) 170 -> 33 us.
 #include <stdint.h>
-
-#include <mutex>
 
 #include "common.h"
 
 namespace dmrg {
 
-constexpr int kW = 4;          // warps per block
-constexpr int kT = 32;         // output tile edge, small-term inner limit
-constexpr int kDepth = 4;      // terms in flight per warp
-constexpr int kRingBytes = 12288;
-constexpr int kXS = kT * (kT + 1);
+namespace {
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void cp_wait_n(int n) {
-  switch (n) {
-    case 0: cp_wait<0>(); break;
-    case 1: cp_wait<1>(); break;
-    case 2: cp_wait<2>(); break;
-    default: cp_wait<3>(); break;
-  }
+constexpr int kT = 32;         // output tile edge, chunk of the inner dimensions
+constexpr int kLd = kT + 1;    // row stride in shared memory: no bank conflicts down a column
+constexpr int kThr = 128;
+constexpr int kSlots = 4;
+// L-first association: terms with inner dimensions up to kT whose three blocks together have at
+// most this many elements (each rounded up to 16 bytes)
+constexpr int kTermMost = 1536;
+
+__device__ __forceinline__ int even(int e) { return (e + 1) & ~1; }
+__device__ __forceinline__ double negate_if(double x, int sign_bit) {
+  return __hiloint2double(__double2hiint(x) ^ sign_bit, __double2loint(x));
 }
 
-template <class T>
-__device__ __forceinline__ int round_vec(int e) {
-  constexpr int v = 16 / int(sizeof(T));
-  return (e + v - 1) / v * v;
-}
-
-// elements a small term occupies in the ring (three 16-byte aligned pieces)
-template <class T>
-__device__ __forceinline__ int term_elems(int m, int n, int dLi, int dRi) {
-  return round_vec<T>(m * dLi) + round_vec<T>(n * dRi) + round_vec<T>(dLi * dRi);
-}
-
-// rows x cols of a row-major source (ld) into dst (leading dimension cols), one
-// asynchronous copy per element (chunk rows need not start on 16-byte boundaries)
-template <class T>
-__device__ __forceinline__ void stage_chunk(T* dst, const T* src, int rows, int cols, int ld,
-                                            int lane) {
-  static_assert(sizeof(T) == 4 || sizeof(T) == 8, "element size");
-  for (int e = lane; e < rows * cols; e += 32) {
-    const int r = e / cols, cc = e - r * cols;
-    const unsigned sm = static_cast<unsigned>(__cvta_generic_to_shared(dst + e));
-    const T* g = src + (int64_t)r * ld + cc;
-    if (sizeof(T) == 8)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sm), "l"(g) : "memory");
-    else
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sm), "l"(g) : "memory");
-  }
-}
-
-template <class T>
-__device__ __forceinline__ void stage(T* dst, const T* src, int elems, int lane) {
-  const int nv = (elems * int(sizeof(T)) + 15) / 16;
-  for (int v = lane; v < nv; v += 32)
-    cp_async16(reinterpret_cast<char*>(dst) + 16 * v, reinterpret_cast<const char*>(src) + 16 * v);
-}
-
-template <class T>
-__global__ void __launch_bounds__(kW * 32, sizeof(T) == 4 ? 4 : 2)
-    k_heff_fused(const HeffTile* __restrict__ tiles, const HeffItem* __restrict__ items,
-                 const HeffPtrs<T> ptrs) {
-  constexpr int kRing = kRingBytes / int(sizeof(T));
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* const base = reinterpret_cast<T*>(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* const ring = base + warp * (kRing + kXS);
-  T* const Xs = ring + kRing;
-  __shared__ int slot_pos[kW][kDepth];
-  const HeffTile t = tiles[blockIdx.x];
+__global__ void __launch_bounds__(kThr, 8)
+k_heff_fused(const HeffTile* __restrict__ tiles, const HeffItem* __restrict__ items,
+             const HeffPtrs<double> ptrs) {
+  __shared__ double Xs[kT * kLd], Rs[kT * kLd], acc[kT * kT];
+  const HeffTile t = tiles[blockIdx.x / kSlots];
+  const int slot = blockIdx.x % kSlots;
   if (ptrs.active && !ptrs.active[t.inst]) return;   // whole block: uniform
-  const T* __restrict__ L = ptrs.L[t.inst];
-  const T* __restrict__ R = ptrs.R[t.inst];
-  const T* __restrict__ X = ptrs.X[t.inst];
-  T* __restrict__ Y = ptrs.Y[t.inst];
-  T* __restrict__ P = ptrs.P[t.inst];
-  const int m = t.m, n = t.n;
-  const int G = 32 / n;                // row groups
-  const int c = lane % n, g = lane / n;
-  const bool act = g < G;
-  const int rows_mine = act ? (m - g + G - 1) / G : 0;   // rows g, g+G, ... < m
-  T acc[kT];
-#pragma unroll
-  for (int q = 0; q < kT; ++q) acc[q] = T(0);
-
-  const int first = t.i0 + warp;
-  const int cnt = first < t.i1 ? (t.i1 - first + kW - 1) / kW : 0;
-  // ring state: terms in flight occupy [headpos, tail) or, once wrapped,
-  // [headpos, end of the used part) and [0, tail)
-  int issued = 0, done = 0, inflight = 0, tail = 0, headpos = 0;
-  bool wrapped = false;
-
-  while (done < cnt) {
-    // prefetch following terms into the ring (circular, in order)
-    while (inflight < kDepth && issued < cnt) {
-      const HeffItem it = items[first + issued * kW];
-      const int S = term_elems<T>(m, n, it.dLi, it.dRi);
-      if (it.dLi > kT || it.dRi > kT || S > kRing) break;
-      int pos;
-      if (inflight == 0) {
-        pos = 0;
-        wrapped = false;
-      } else if (!wrapped) {
-        if (tail + S <= kRing) {
-          pos = tail;
-        } else if (S <= headpos) {
-          pos = 0;
-          wrapped = true;
-        } else {
-          break;
-        }
-      } else {
-        if (tail + S <= headpos) pos = tail;
-        else break;
-      }
-      T* dst = ring + pos;
-      stage(dst, L + it.loff + (int64_t)t.r0 * it.dLi, m * it.dLi, lane);
-      dst += round_vec<T>(m * it.dLi);
-      stage(dst, R + it.roff + (int64_t)t.c0 * it.dRi, n * it.dRi, lane);
-      dst += round_vec<T>(n * it.dRi);
-      stage(dst, X + it.xoff, it.dLi * it.dRi, lane);
-      cp_commit();
-      if (lane == 0) slot_pos[warp][issued % kDepth] = pos;
-      if (inflight == 0) headpos = pos;
-      tail = pos + S;
-      ++issued;
-      ++inflight;
-    }
-    const HeffItem it = items[first + done * kW];
-    const T sg = T(it.sign);
+  const double* __restrict__ L = ptrs.L[t.inst];
+  const double* __restrict__ R = ptrs.R[t.inst];
+  const double* __restrict__ X = ptrs.X[t.inst];
+  const int tid = threadIdx.x;
+  const int m = t.m, n = t.n, mn = m * n;
+  const int inv_n = 65536 / n + 1;   // e / n = (e inv_n) >> 16 for e < 1024, n <= 32
+  for (int e = tid; e < mn; e += kThr) acc[e] = 0.0;   // (read by the same thread only)
+  for (int j = t.i0 + slot; j < t.i1; j += kSlots) {
+    const HeffItem it = items[j];
     const int dLi = it.dLi, dRi = it.dRi;
-    if (inflight == 0) {
-      // large term: chunks staged into the (empty) ring by asynchronous copies; X rows
-      // accumulate in shared memory over the chunks of the psi columns (same order of
-      // summation as a single pass)
-      ++issued;
-      constexpr int KC = kRing / (3 * kT) < kT ? kRing / (3 * kT) : kT;   // rows per chunk
-      T* const Pc = ring;              // psi chunk (kc x rc), then the L chunk (m x kc)
-      T* const Rc = ring + KC * kT;    // R chunk (n x rc)
-      for (int k0 = 0; k0 < dLi; k0 += KC) {
-        const int kc = min(KC, dLi - k0);
-        for (int r0 = 0; r0 < dRi; r0 += kT) {
-          const int rc = min(kT, dRi - r0);
-          stage_chunk(Pc, X + it.xoff + (int64_t)k0 * dRi + r0, kc, rc, dRi, lane);
-          stage_chunk(Rc, R + it.roff + (int64_t)t.c0 * dRi + r0, n, rc, dRi, lane);
-          cp_commit();
-          cp_wait<0>();
-          __syncwarp();
-          if (act) {
-            const T* rr = Rc + c * rc;
-            for (int i = g; i < kc; i += G) {
-              const T* pr = Pc + i * rc;
-              T s = r0 ? Xs[i * (kT + 1) + c] : T(0);
-              for (int r = 0; r < rc; ++r) s = fma(pr[r], rr[r], s);
-              Xs[i * (kT + 1) + c] = s;
-            }
-          }
-          __syncwarp();
-        }
-        stage_chunk(Pc, L + it.loff + (int64_t)t.r0 * dLi + k0, m, kc, dLi, lane);
-        cp_commit();
-        cp_wait<0>();
-        __syncwarp();
-        if (act) {
-          const T* lr = Pc + g * kc;
-          for (int k = 0; k < kc; ++k) {
-            const T xv = sg * Xs[k * (kT + 1) + c];
-#pragma unroll
-            for (int q = 0; q < kT; ++q)
-              if (q < rows_mine) acc[q] = fma(lr[q * G * kc + k], xv, acc[q]);
-          }
-        }
-        __syncwarp();
+    const int neg = it.sign < 0.f ? int(0x80000000) : 0;
+    const double* __restrict__ Lb = L + it.loff + int64_t(t.r0) * dLi;
+    const double* __restrict__ Rb = R + it.roff + int64_t(t.c0) * dRi;
+    const double* __restrict__ Pb = X + it.xoff;
+    if (dLi <= kT && dRi <= kT && even(m * dLi) + even(n * dRi) + even(dLi * dRi) <= kTermMost &&
+        int64_t(m) * dRi * (dLi + n) < int64_t(n) * dLi * (dRi + m)) {
+      // Z = L psi (m x dRi), then acc += Z (s R)^T
+      const int inv_r = 65536 / dRi + 1;
+      for (int e = tid; e < n * dRi; e += kThr) {
+        const int c = (e * inv_r) >> 16, b = e - c * dRi;
+        Rs[c * kLd + b] = negate_if(Rb[e], neg);
       }
-      ++done;
+      for (int e = tid; e < m * dRi; e += kThr) {
+        const int i = (e * inv_r) >> 16, b = e - i * dRi;
+        const double* lr = Lb + i * dLi;
+        const double* pr = Pb + b;
+        double s = 0.0;
+#pragma unroll 4
+        for (int a = 0; a < dLi; ++a) s = fma(lr[a], pr[a * dRi], s);
+        Xs[i * kLd + b] = s;
+      }
+      __syncthreads();
+      for (int e = tid; e < mn; e += kThr) {
+        const int i = (e * inv_n) >> 16, c = e - i * n;
+        const double* zr = Xs + i * kLd;
+        const double* rr = Rs + c * kLd;
+        double a = acc[e];
+#pragma unroll 4
+        for (int b = 0; b < dRi; ++b) a = fma(zr[b], rr[b], a);
+        acc[e] = a;
+      }
+      __syncthreads();
       continue;
     }
-    // wait for the oldest term in flight (later groups may still be pending)
-    cp_wait_n(inflight - 1);
-    __syncwarp();
-    const T* Ls = ring + slot_pos[warp][done % kDepth];
-    const T* Rs = Ls + round_vec<T>(m * dLi);
-    const T* Ps = Rs + round_vec<T>(n * dRi);
-    // the cheaper association of L psi R^T for this tile: (psi R^T) first or (L psi) first
-    const bool lfirst = int64_t(m) * dRi * (dLi + n) < int64_t(n) * dLi * (dRi + m);
-    if (!lfirst) {
-      if (act) {
-        const T* rr = Rs + c * dRi;
-        for (int i = g; i < dLi; i += G) {
-          const T* pr = Ps + i * dRi;
-          T s = T(0);
-          for (int r = 0; r < dRi; ++r) s = fma(pr[r], rr[r], s);
-          Xs[i * (kT + 1) + c] = s;
+    for (int k0 = 0; k0 < dLi; k0 += kT) {
+      const int kc = min(kT, dLi - k0);
+      for (int r0 = 0; r0 < dRi; r0 += kT) {
+        const int rc = min(kT, dRi - r0);
+        // columns of the R tile: a warp reads rows of rc consecutive elements
+        if (k0 == 0 || dRi > kT) {
+          if (rc == dRi) {
+            const int inv_r = 65536 / rc + 1;
+            for (int e = tid; e < n * rc; e += kThr) {
+              const int c = (e * inv_r) >> 16, b = e - c * rc;
+              Rs[c * kLd + b] = Rb[e];
+            }
+          } else {
+            for (int e = tid; e < n * kT; e += kThr) {
+              const int c = e >> 5, b = e & 31;
+              if (b < rc) Rs[c * kLd + b] = Rb[int64_t(c) * dRi + r0 + b];
+            }
+          }
+          __syncthreads();
         }
-      }
-      __syncwarp();
-      if (act) {
-        const T* lr = Ls + g * dLi;
-        for (int k = 0; k < dLi; ++k) {
-          const T xv = sg * Xs[k * (kT + 1) + c];
-#pragma unroll
-          for (int q = 0; q < kT; ++q)
-            if (q < rows_mine) acc[q] = fma(lr[q * G * dLi + k], xv, acc[q]);
+        const bool last = r0 + kT >= dRi;
+        for (int e = tid; e < kc * n; e += kThr) {
+          const int i = (e * inv_n) >> 16, c = e - i * n;
+          const double* pr = Pb + int64_t(k0 + i) * dRi + r0;
+          const double* rr = Rs + c * kLd;
+          double s = r0 ? Xs[i * kLd + c] : 0.0;
+#pragma unroll 4
+          for (int r = 0; r < rc; ++r) s = fma(pr[r], rr[r], s);
+          Xs[i * kLd + c] = last ? negate_if(s, neg) : s;
         }
+        __syncthreads();
       }
-    } else {
-      // Z (m x dRi) = L psi in shared memory, then acc[i][c] += s sum_b Z[i][b] R[c][b]
-      for (int e = lane; e < m * dRi; e += 32) {
-        const int i = e / dRi, b = e - i * dRi;
-        const T* lr = Ls + i * dLi;
-        T s = T(0);
-        for (int a = 0; a < dLi; ++a) s = fma(lr[a], Ps[a * dRi + b], s);
-        Xs[i * (kT + 1) + b] = s;
+      for (int e = tid; e < mn; e += kThr) {
+        const int i = (e * inv_n) >> 16, c = e - i * n;
+        const double* lr = Lb + int64_t(i) * dLi + k0;
+        const double* xr = Xs + c;
+        double a = acc[e];
+#pragma unroll 4
+        for (int k = 0; k < kc; ++k) a = fma(lr[k], xr[k * kLd], a);
+        acc[e] = a;
       }
-      __syncwarp();
-      if (act) {
-        const T* rr = Rs + c * dRi;
-        for (int b = 0; b < dRi; ++b) {
-          const T rv = sg * rr[b];
-#pragma unroll
-          for (int q = 0; q < kT; ++q)
-            if (q < rows_mine) acc[q] = fma(Xs[(g + q * G) * (kT + 1) + b], rv, acc[q]);
-        }
-      }
-    }
-    __syncwarp();
-    ++done;
-    --inflight;
-    if (inflight > 0) {
-      const int np = slot_pos[warp][done % kDepth];
-      if (np < headpos) wrapped = false;   // the head crossed into the wrapped part
-      headpos = np;
-    } else {
-      tail = headpos = 0;
-      wrapped = false;
+      __syncthreads();
     }
   }
-  cp_wait<0>();
-  // fixed-order reduction of the warps' partial tiles (reuses the rings)
-  __syncthreads();
-  T* const red = base + warp * (kRing + kXS);
-  if (act) {
+  double* __restrict__ P = ptrs.P[t.inst] + t.qoff + int64_t(slot) * mn;
+  for (int e = tid; e < mn; e += kThr) P[e] = acc[e];
+}
+
+// psi' tile = sum over groups (in group order) of the partial tiles, each the sum of its slots
+// in order: red[0 .. n_plain) have one partial tile per group (poff; the small-block kernel),
+// the others four (qoff)
+__global__ void __launch_bounds__(128)
+k_heff_reduce_slots(const HeffRed* __restrict__ red, int64_t n_plain, const HeffPtrs<double> ptrs) {
+  const HeffRed r = red[blockIdx.x];
+  if (ptrs.active && !ptrs.active[r.inst]) return;
+  const bool plain = blockIdx.x < n_plain;
+  const double* __restrict__ P = ptrs.P[r.inst] + (plain ? r.poff : r.qoff);
+  double* __restrict__ Y = ptrs.Y[r.inst];
+  const int mn = r.m * r.n;
+  for (int e = threadIdx.x; e < mn; e += blockDim.x) {
+    double s = 0.0;
+    for (int g = 0; g < r.groups; ++g) {
+      if (plain) {
+        s += P[int64_t(g) * mn + e];
+      } else {
+        const double* q = P + int64_t(g) * kSlots * mn + e;
+        double u = q[0];
 #pragma unroll
-    for (int q = 0; q < kT; ++q)
-      if (q < rows_mine) red[(g + q * G) * n + c] = acc[q];
-  }
-  __syncthreads();
-  const int mn = m * n;
-  for (int e = threadIdx.x; e < mn; e += kW * 32) {
-    T s = base[e];
-#pragma unroll
-    for (int w = 1; w < kW; ++w) s += base[w * (kRing + kXS) + e];
-    if (t.poff < 0) {
-      const int i = e / n, cc = e - i * n;
-      Y[t.yoff + (int64_t)(t.r0 + i) * t.ld + t.c0 + cc] = s;
-    } else {
-      P[t.poff + e] = s;
+        for (int w = 1; w < kSlots; ++w) u += q[int64_t(w) * mn];
+        s = r.groups > 1 ? s + u : u;
+      }
     }
+    const int i = e / r.n, c = e - i * r.n;
+    Y[r.yoff + int64_t(r.r0 + i) * r.ld + r.c0 + c] = s;
   }
 }
+
+}  // namespace
 
 // psi' tile = sum over groups (in group order) of the partial tiles
 template <class T>
@@ -320,23 +210,18 @@ void heff_reduce(const HeffRed* d_red, int64_t n_red, const HeffPtrs<T>& ptrs, c
 template void heff_reduce<float>(const HeffRed*, int64_t, const HeffPtrs<float>&, cudaStream_t);
 template void heff_reduce<double>(const HeffRed*, int64_t, const HeffPtrs<double>&, cudaStream_t);
 
-template <class T>
-void heff_fused(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
-                const HeffRed* d_red, int64_t n_red, const HeffPtrs<T>& ptrs, cudaStream_t s) {
+void heff_fused64(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
+                  const HeffRed* d_red, int64_t n_plain, int64_t n_red,
+                  const HeffPtrs<double>& ptrs, cudaStream_t s) {
   if (n_tiles > 0) {
-    const size_t smem = sizeof(T) * kW * (kRingBytes / sizeof(T) + kXS);
-    static std::once_flag attr_once;   // per process: the attribute belongs to the kernel
-    std::call_once(attr_once, [&] {
-      DMRG_CUDA(cudaFuncSetAttribute(k_heff_fused<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     int(smem)));
-    });
-    k_heff_fused<T><<<int(n_tiles), kW * 32, smem, s>>>(d_tiles, d_items, ptrs);
+    k_heff_fused<<<int(n_tiles * kSlots), kThr, 0, s>>>(d_tiles, d_items, ptrs);
     DMRG_LAUNCHED();
   }
-  heff_reduce<T>(d_red, n_red, ptrs, s);   // partial tiles of both product kernels
+  if (n_red > 0) {
+    k_heff_reduce_slots<<<int(n_red), 128, 0, s>>>(d_red, n_plain, ptrs);
+    DMRG_LAUNCHED();
+  }
 }
-template void heff_fused<double>(const HeffTile*, int64_t, const HeffItem*, const HeffRed*,
-                                 int64_t, const HeffPtrs<double>&, cudaStream_t);
 
 // staging with the vector pointer read from device memory (graph replay on new vectors)
 template <class TO>
