@@ -283,16 +283,18 @@ struct TaskList {
   void clear() { tasks.clear(); terms.clear(); }
 };
 
-// device-resident, split into small (warp per task) and large (tiled) parts
+// device-resident, split into small (units of 32 outputs) and large (tiled) parts
 struct DevTaskList {
   DevBuf<GemmTask> small_tasks, large_tasks;
   DevBuf<GemmTerm> terms;
   DevBuf<GemmTile> tiles;
-  int64_t n_small = 0, n_large = 0, n_tiles = 0;
+  DevBuf<GemmTile> units;   // 32 outputs of a small task: task, first output (m0)
+  int64_t n_small = 0, n_large = 0, n_tiles = 0, n_units = 0;
+  bool many_terms = false;  // some small task sums over many terms
   double flops = 0;      // algorithmic flops of the list
   // base_elems[b]: elements addressable through base b (0 = unused); every operand range
   // is checked against it on the host before the list reaches the device
-  // small_limit: tasks of at most this many outputs run one warp each; the others are cut
+  // small_limit: tasks of at most this many outputs run in units of 32; the others are cut
   // into 64 x 64 tiles (0: every task tiled, the form the tensor-core engine wants)
   void build(const TaskList& L, const int64_t* base_elems, cudaStream_t s,
              int64_t small_limit = 1024);

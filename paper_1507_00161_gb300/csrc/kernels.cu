@@ -2,8 +2,8 @@
 //
 //  * task-list GEMMs: C (M x N) (+)= sum_t alpha_t op(A_t) op(B_t) over thousands of small
 //    per-sector blocks (superblock product, reduced density matrices, renormalization,
-//    wave-function transformation).  Tiny tasks run one per warp straight from L1/L2;
-//    large tasks are cut into 64 x 64 tiles staged through shared memory.
+//    wave-function transformation).  Small tasks run in units of 32 outputs straight from
+//    L1/L2; large tasks are cut into 64 x 64 tiles staged through shared memory.
 //  * copy tasks: scaled sums of operator blocks into enlarged-operator sub-blocks.
 //  * vector kernels with deterministic (fixed-order) reductions (the chain of a Davidson
 //    iteration: davidson.cu).
@@ -28,7 +28,16 @@ std::atomic<int64_t> g_malloc_count{0}, g_malloc_ns{0};
 constexpr int kWarp = 32;
 
 // ------------------------------------------------------------------------------------
-// task-list GEMM, one warp per task
+// task-list GEMM, small tasks, in units of 32 outputs of a task (GemmTile: task, first output).
+// An FP64 multiply-add takes 64 clocks however few of its lanes are used, so a sum of K products
+// is a chain of 64 K clocks for whoever forms it: a whole task per warp (as many chains one after
+// the other as it has 32 outputs) left the superblock products of narrow blocks at 1 ms for 4
+// MFLOP.  Every output is  sum_t alpha_t (sum_k A_t B_t)  in term order, the inner sums first:
+//   - k_gemm_small: one warp per unit;
+//   - k_gemm_small_terms, for lists whose tasks sum over many terms: the inner sums do not
+//     depend on each other, so seven warps form them, 28 terms at a time, and the eighth adds
+//     the previous 28 in order.
+// Measured (GB300), pf 4p+4n at position 6, M0 = 1024, the two passes of the product: 715 -> 48 us.
 // ------------------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ T ld_op(const T* base, int trans, int ld, int r, int c) {
@@ -36,33 +45,83 @@ __device__ __forceinline__ T ld_op(const T* base, int trans, int ld, int r, int 
   return trans ? base[(int64_t)c * ld + r] : base[(int64_t)r * ld + c];
 }
 
+// sum over k of one term's products for output (m, n)
 template <class T>
-__global__ void __launch_bounds__(256) k_gemm_small(const GemmTask* __restrict__ tasks,
-                                                    int64_t n_tasks,
+__device__ __forceinline__ T term_sum(const GemmTerm& g, const Bases<T>& b, int m, int n) {
+  const T* A = b.p[g.A.base] + g.A.off;
+  const T* B = b.p[g.B.base] + g.B.off;
+  const int ta = g.trans & 1, tb = (g.trans >> 1) & 1;
+  const T* pa = ta ? A + m : A + int64_t(m) * g.A.ld;
+  const T* pb = tb ? B + int64_t(n) * g.B.ld : B + n;
+  const int64_t sa = ta ? g.A.ld : 1, sb = tb ? 1 : g.B.ld;
+  T s = T(0);
+#pragma unroll 4
+  for (int k = 0; k < g.K; ++k) s = fma(pa[k * sa], pb[k * sb], s);
+  return s;
+}
+
+template <class T>
+__global__ void __launch_bounds__(256) k_gemm_small(const GemmTile* __restrict__ units,
+                                                    int64_t n_units,
+                                                    const GemmTask* __restrict__ tasks,
                                                     const GemmTerm* __restrict__ terms,
                                                     Bases<T> b, int beta_zero,
                                                     const int32_t* __restrict__ active) {
   if (active && !active[0]) return;
-  int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / kWarp;
-  int lane = threadIdx.x & (kWarp - 1);
-  if (w >= n_tasks) return;
-  const GemmTask t = tasks[w];
-  T* C = b.p[t.C.base] + t.C.off;
-  const int MN = t.M * t.N;
-  for (int idx = lane; idx < MN; idx += kWarp) {
-    const int m = idx / t.N, n = idx - m * t.N;
-    T acc = T(0);
-    for (int j = t.t0; j < t.t1; ++j) {
-      const GemmTerm g = terms[j];
-      const T* A = b.p[g.A.base] + g.A.off;
-      const T* B = b.p[g.B.base] + g.B.off;
-      const int ta = g.trans & 1, tb = (g.trans >> 1) & 1;
-      T s = T(0);
-      for (int k = 0; k < g.K; ++k)
-        s = fma(ld_op(A, ta, g.A.ld, m, k), ld_op(B, tb, g.B.ld, k, n), s);
-      acc = fma(T(g.alpha), s, acc);
+  const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / kWarp;
+  const int lane = threadIdx.x & (kWarp - 1);
+  if (w >= n_units) return;
+  const GemmTile u = units[w];
+  const GemmTask t = tasks[u.task];
+  const int idx = u.m0 + lane;
+  if (idx >= t.M * t.N) return;
+  const int m = idx / t.N, n = idx - m * t.N;
+  T acc = T(0);
+  for (int j = t.t0; j < t.t1; ++j) {
+    const GemmTerm g = terms[j];
+    acc = fma(T(g.alpha), term_sum<T>(g, b, m, n), acc);
+  }
+  T* c = b.p[t.C.base] + t.C.off + (int64_t)m * t.C.ld + n;
+  *c = beta_zero ? acc : (*c + acc);
+}
+
+constexpr int kSumWarps = 7, kSumPer = 4, kSumTerms = kSumWarps * kSumPer;
+
+template <class T>
+__global__ void __launch_bounds__(256) k_gemm_small_terms(const GemmTile* __restrict__ units,
+                                                          const GemmTask* __restrict__ tasks,
+                                                          const GemmTerm* __restrict__ terms,
+                                                          Bases<T> b, int beta_zero,
+                                                          const int32_t* __restrict__ active) {
+  if (active && !active[0]) return;
+  __shared__ T sum[2][kSumTerms][kWarp];
+  __shared__ T alpha[2][kSumTerms];
+  const GemmTile u = units[blockIdx.x];
+  const GemmTask t = tasks[u.task];
+  const int warp = threadIdx.x / kWarp, lane = threadIdx.x & (kWarp - 1);
+  const int idx = u.m0 + lane;
+  const bool on = idx < t.M * t.N;
+  const int m = idx / t.N, n = idx - m * t.N;
+  T acc = T(0);
+  int buf = 0, before = 0;   // terms of the other buffer still to be added
+  for (int j0 = t.t0; j0 < t.t1 || before; j0 += kSumTerms) {
+    if (warp == 0) {
+      for (int x = 0; x < before; ++x) acc = fma(alpha[buf ^ 1][x], sum[buf ^ 1][x][lane], acc);
+    } else {
+      for (int y = 0; y < kSumPer; ++y) {
+        const int x = warp - 1 + kSumWarps * y;
+        if (j0 + x >= t.t1) break;
+        const GemmTerm g = terms[j0 + x];
+        sum[buf][x][lane] = on ? term_sum<T>(g, b, m, n) : T(0);
+        if (lane == 0) alpha[buf][x] = T(g.alpha);
+      }
     }
-    T* c = C + (int64_t)m * t.C.ld + n;
+    before = max(0, min(kSumTerms, t.t1 - j0));
+    buf ^= 1;
+    __syncthreads();
+  }
+  if (warp == 0 && on) {
+    T* c = b.p[t.C.base] + t.C.off + (int64_t)m * t.C.ld + n;
     *c = beta_zero ? acc : (*c + acc);
   }
 }
@@ -84,6 +143,10 @@ __global__ void __launch_bounds__(256) k_gemm_tiled(const GemmTile* __restrict__
   const GemmTile tl = tiles[blockIdx.x];
   const GemmTask t = tasks[tl.task];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  // rows ty + 16 i and columns tx + 16 j inside the task, by warp (padding costs as much FP64
+  // time as work: a 40 x 40 task is 1600 of 4096 outputs)
+  const int ni = min(4, max(0, t.M - tl.m0 - 2 * int(threadIdx.x >> 5) + 15) >> 4);
+  const int nj = min(4, (t.N - tl.n0 + 15) >> 4);
   T acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -107,8 +170,8 @@ __global__ void __launch_bounds__(256) k_gemm_tiled(const GemmTile* __restrict__
         Bs[kk][nn] = (gn < t.N && gk < g.K) ? ld_op(B, tb, g.B.ld, gk, gn) : T(0);
       }
       __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < TK; ++kk) {
+      const int kn = min(TK, g.K - k0);
+      for (int kk = 0; kk < kn; ++kk) {
         T a[4], bb[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
@@ -116,8 +179,10 @@ __global__ void __launch_bounds__(256) k_gemm_tiled(const GemmTile* __restrict__
         for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
+          if (i < ni)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+            for (int j = 0; j < 4; ++j)
+              if (j < nj) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
       }
       __syncthreads();
     }
@@ -171,12 +236,15 @@ void DevTaskList::build(const TaskList& L, const int64_t* be, cudaStream_t s,
     }
   }
   std::vector<GemmTask> sm, lg;
-  std::vector<GemmTile> tl;
+  std::vector<GemmTile> tl, un;
   flops = 0;
+  many_terms = false;
   for (const auto& t : L.tasks) {
     for (int j = t.t0; j < t.t1; ++j) flops += 2.0 * t.M * t.N * double(L.terms[j].K);
     if (t.M <= 0 || t.N <= 0) continue;
     if (int64_t(t.M) * t.N <= small_limit) {
+      for (int i = 0; i < t.M * t.N; i += kWarp) un.push_back(GemmTile{int(sm.size()), i, 0});
+      many_terms = many_terms || t.t1 - t.t0 >= kSumWarps;
       sm.push_back(t);
     } else {
       int id = int(lg.size());
@@ -186,6 +254,8 @@ void DevTaskList::build(const TaskList& L, const int64_t* be, cudaStream_t s,
     }
   }
   small_tasks.upload(sm, s);
+  units.upload(un, s);
+  n_units = int64_t(un.size());
   large_tasks.upload(lg, s);
   tiles.upload(tl, s);
   terms.upload(L.terms, s);
@@ -197,11 +267,13 @@ void DevTaskList::build(const TaskList& L, const int64_t* be, cudaStream_t s,
 template <class T>
 void run_gemm_tasks(const DevTaskList& L, const Bases<T>& b, int beta_zero, cudaStream_t s,
                     const int32_t* active) {
-  if (L.n_small) {
-    int64_t threads = L.n_small * kWarp;
-    int blocks = int((threads + 255) / 256);
-    k_gemm_small<T><<<blocks, 256, 0, s>>>(L.small_tasks.p, L.n_small, L.terms.p, b, beta_zero,
-                                           active);
+  if (L.n_units && L.many_terms) {
+    k_gemm_small_terms<T><<<int(L.n_units), 256, 0, s>>>(L.units.p, L.small_tasks.p, L.terms.p, b,
+                                                         beta_zero, active);
+    DMRG_LAUNCHED();
+  } else if (L.n_units) {
+    k_gemm_small<T><<<int((L.n_units + 7) / 8), 256, 0, s>>>(L.units.p, L.n_units, L.small_tasks.p,
+                                                             L.terms.p, b, beta_zero, active);
     DMRG_LAUNCHED();
   }
   if (L.n_tiles) {
