@@ -3,15 +3,19 @@
 // dimensions and whose terms' inner dimensions are all at most 16.
 //
 // At large M the sector count grows with M, so most wave-function blocks are a few states
-// on a side: a term is a handful of multiply-adds and the work is streaming the operator
-// blocks.  One warp per (output block, group of at most 16 terms), plain FMAs on the CUDA
-// cores, operands read through the L1 (no staging, no padding to matrix-instruction shapes).
-// Lane map for an m x n output block: column c = lane mod n, row group g = lane / n,
-// G = floor(32 / n) groups; per term
-//     X[a][c] = sum_b psi[a][b] R[c][b]   (rows a = g, g + G, ...; X in shared memory)
-//     acc[i][c] += s sum_a L[i][a] X[a][c] (rows i = g, g + G, ...; acc in registers)
-// Terms are added in list order; groups of one block are added in group order by
-// k_heff_reduce: the result is deterministic.
+// on a side: a term is a handful of multiply-adds, and a warp that takes the terms one after the
+// other waits for its loads (descriptor, psi and R, L) at every one of them.  The terms of a
+// group only meet in the sum  acc <- acc + s_k (L_k X_k),  so one thread block takes an (output
+// block, group of at most 16 terms): its warps form the products  D_k = L_k (psi R_k^T)  of
+// different terms side by side and leave them in shared memory, then the block adds them in term
+// order.  Lane map for an m x n output block: elements are numbered through and dealt to the
+// lanes 32 at a time (an FP64 instruction takes as long with half of its lanes); per term
+//     X[a][c] = sum_b psi[a][b] R[c][b]     (X in shared memory, per warp)
+//     D[i][c] = sum_a L[i][a] X[a][c]
+// Terms are added in list order; groups of one block are added in group order by the
+// reduction kernels: the result is deterministic.
+// Measured (GB300) against one warp per group, FP32: pf 4p+5n, M0 = 777 (615 groups) 16.8 -> 4.7 us,
+// pf 8p+8n at M = 4096, position 15 (1135 groups) 20.6 -> 7.9 us.
 #include <stdint.h>
 
 #include "common.h"
@@ -21,83 +25,61 @@ namespace dmrg {
 namespace {
 
 constexpr int kSmWarps = 8;
+constexpr int kSmTerms = 16;   // most terms of a group
 
 template <class T>
-__global__ void __launch_bounds__(kSmWarps * 32, 3)
-k_heff_small(const HeffTile* __restrict__ tiles, int64_t n_tiles,
-             const HeffItem* __restrict__ items, const HeffPtrs<T> ptrs) {
-  __shared__ T Xs[kSmWarps][kSmallEdge * kSmallEdge];
+__global__ void __launch_bounds__(kSmWarps * 32)
+k_heff_small(const HeffTile* __restrict__ tiles, const HeffItem* __restrict__ items,
+             const HeffPtrs<T> ptrs) {
+  constexpr int kE = kSmallEdge * kSmallEdge;
+  __shared__ T Xs[kSmWarps][kE];
+  extern __shared__ __align__(16) unsigned char small_sm[];
+  T* const D = reinterpret_cast<T*>(small_sm);   // products of the terms, m n elements each
+  const HeffTile t = tiles[blockIdx.x];
+  if (ptrs.active && !ptrs.active[t.inst]) return;
+  const T* __restrict__ L = ptrs.L[t.inst];
+  const T* __restrict__ R = ptrs.R[t.inst];
+  const T* __restrict__ X = ptrs.X[t.inst];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m = t.m, n = t.n, mn = m * n;
+  const int inv_n = 65536 / n + 1;   // e / n = (e inv_n) >> 16 for e < 256
   T* Xw = Xs[warp];
-  for (int64_t w = int64_t(blockIdx.x) * kSmWarps + warp; w < n_tiles;
-       w += int64_t(gridDim.x) * kSmWarps) {
-    const HeffTile t = tiles[w];
-    if (ptrs.active && !ptrs.active[t.inst]) continue;
-    const T* __restrict__ L = ptrs.L[t.inst];
-    const T* __restrict__ R = ptrs.R[t.inst];
-    const T* __restrict__ X = ptrs.X[t.inst];
-    const int m = t.m, n = t.n;
-    const int G = 32 / n;
-    const int c = lane % n, g = lane / n;
-    const bool on = g < G;
-    T acc[kSmallEdge / 2];
-#pragma unroll
-    for (int q = 0; q < kSmallEdge / 2; ++q) acc[q] = T(0);
-    for (int base = t.i0; base < t.i1; base += 32) {
-      // the lanes load the next 32 term descriptors at once; each term broadcasts its own
-      HeffItem mine{};
-      if (base + lane < t.i1) mine = items[base + lane];
-      const int cnt = min(32, t.i1 - base);
-      for (int j = 0; j < cnt; ++j) {
-        const int64_t loff = __shfl_sync(0xffffffffu, (long long)mine.loff, j);
-        const int64_t roff = __shfl_sync(0xffffffffu, (long long)mine.roff, j);
-        const int64_t xoff = __shfl_sync(0xffffffffu, (long long)mine.xoff, j);
-        const int dLi = __shfl_sync(0xffffffffu, mine.dLi, j);
-        const int dRi = __shfl_sync(0xffffffffu, mine.dRi, j);
-        const float sign = __shfl_sync(0xffffffffu, mine.sign, j);
-        const T* __restrict__ Lb = L + loff + int64_t(t.r0) * dLi;
-        const T* __restrict__ Rb = R + roff + int64_t(t.c0 + c) * dRi;
-        const T* __restrict__ Xb = X + xoff;
-        if (on) {
-          for (int a = g; a < dLi; a += G) {
-            T s = T(0);
-            for (int b = 0; b < dRi; ++b) s = fma(Xb[a * dRi + b], Rb[b], s);
-            Xw[a * n + c] = s;
-          }
-        }
-        __syncwarp();
-        if (on) {
-          const T sg = T(sign);
-#pragma unroll
-          for (int q = 0; q < kSmallEdge / 2; ++q) {
-            const int i = g + q * G;
-            if (i < m) {
-              T s = T(0);
-              for (int a = 0; a < dLi; ++a) s = fma(Lb[i * dLi + a], Xw[a * n + c], s);
-              acc[q] = fma(sg, s, acc[q]);
-            }
-          }
-        }
-        __syncwarp();
-      }
+  const int cnt = t.i1 - t.i0;
+  for (int j = warp; j < cnt; j += kSmWarps) {
+    const HeffItem it = items[t.i0 + j];
+    const int dLi = it.dLi, dRi = it.dRi;
+    const T* __restrict__ Lb = L + it.loff + int64_t(t.r0) * dLi;
+    const T* __restrict__ Rb = R + it.roff + int64_t(t.c0) * dRi;
+    const T* __restrict__ Xb = X + it.xoff;
+    for (int e = lane; e < dLi * n; e += 32) {
+      const int a = (e * inv_n) >> 16, c = e - a * n;
+      const T* xr = Xb + a * dRi;
+      const T* rr = Rb + c * dRi;
+      T s = T(0);
+#pragma unroll 4
+      for (int b = 0; b < dRi; ++b) s = fma(xr[b], rr[b], s);
+      Xw[e] = s;
     }
-    if (on) {
-      if (t.poff < 0) {
-        T* __restrict__ Y = ptrs.Y[t.inst] + t.yoff;
-#pragma unroll
-        for (int q = 0; q < kSmallEdge / 2; ++q) {
-          const int i = g + q * G;
-          if (i < m) Y[int64_t(t.r0 + i) * t.ld + t.c0 + c] = acc[q];
-        }
-      } else {
-        T* __restrict__ P = ptrs.P[t.inst] + t.poff;
-#pragma unroll
-        for (int q = 0; q < kSmallEdge / 2; ++q) {
-          const int i = g + q * G;
-          if (i < m) P[i * n + c] = acc[q];
-        }
-      }
+    __syncwarp();
+    for (int e = lane; e < mn; e += 32) {
+      const int i = (e * inv_n) >> 16, c = e - i * n;
+      const T* lr = Lb + i * dLi;
+      T s = T(0);
+#pragma unroll 4
+      for (int a = 0; a < dLi; ++a) s = fma(lr[a], Xw[a * n + c], s);
+      D[j * mn + e] = it.sign < 0.f ? -s : s;
     }
+    __syncwarp();
+  }
+  __syncthreads();
+  T* __restrict__ Y = t.poff < 0 ? ptrs.Y[t.inst] + t.yoff + int64_t(t.r0) * t.ld + t.c0
+                                 : ptrs.P[t.inst] + t.poff;
+  const int ld = t.poff < 0 ? t.ld : n;
+  for (int e = threadIdx.x; e < mn; e += kSmWarps * 32) {
+    T acc = T(0);
+    for (int j = 0; j < cnt; ++j) acc += D[j * mn + e];
+    const int i = (e * inv_n) >> 16, c = e - i * n;
+    Y[int64_t(i) * ld + c] = acc;
   }
 }
 
@@ -107,8 +89,8 @@ template <class T>
 void heff_small(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
                 const HeffPtrs<T>& ptrs, cudaStream_t s) {
   if (n_tiles <= 0) return;
-  const int64_t blocks = std::min<int64_t>((n_tiles + kSmWarps - 1) / kSmWarps, 152 * 8 * 16);
-  k_heff_small<T><<<int(blocks), kSmWarps * 32, 0, s>>>(d_tiles, n_tiles, d_items, ptrs);
+  const size_t smem = sizeof(T) * kSmTerms * kSmallEdge * kSmallEdge;
+  k_heff_small<T><<<int(n_tiles), kSmWarps * 32, smem, s>>>(d_tiles, d_items, ptrs);
   DMRG_LAUNCHED();
 }
 template void heff_small<float>(const HeffTile*, int64_t, const HeffItem*, const HeffPtrs<float>&,
