@@ -330,6 +330,19 @@ void run_gemm_tasks(const DevTaskList& L, const Bases<T>& b, int beta_zero, cuda
 template <class TA, class TB, class TC>
 void run_gemm_tasks_tc(const DevTaskList& L, const Bases<void>& b, int beta_zero, cudaStream_t s,
                        const int32_t* active = nullptr);
+// one dense product C (M x N) = op(A) op(B) with the same split-TF32 arithmetic (tgemm.cu);
+// K in `splits` parts of k_len, part z written to C + z c_split.  bias_relu: max(0, . + side[n]);
+// mask: zero where side (laid out as C) is not positive; both with one split
+enum class DenseEpilogue { none, bias_relu, mask };
+struct DenseGemm {
+  const float *A, *B;
+  float* C;
+  const float* side;
+  int32_t M, N, K, lda, ldb, ldc, trans;   // trans as GemmTerm
+  int32_t k_len;
+  int64_t c_split;
+};
+void dense_gemm_tc(const DenseGemm& d, DenseEpilogue e, int splits, cudaStream_t s);
 template <class T>
 void run_copy_tasks(const CopyTask* d_tasks, int64_t n_tasks, const CopyTerm* d_terms,
                     const Bases<T>& b, cudaStream_t s);
@@ -562,17 +575,19 @@ void enlarge_blocks(const EnlBlock* blocks, int64_t n, const int32_t* eptr, cons
 // learned preconditioner (mlp.cu)
 template <class T>
 struct MlpActs {
-  DevBuf<T> Z1, H1, Z2, H2, Z3, H3, Y, dY, dH, dZ;
+  DevBuf<T> Z1, H1, Z2, H2, Z3, H3, Y, dY, dH, dZ, sums;
   DevBuf<double> part;
   int64_t cap = 0;
   void ensure(int64_t B) {
     if (B <= cap) return;
     const int64_t nh = B * 256;
-    Z1.alloc(nh);
+    if (sizeof(T) == 8) {   // the FP32 network masks by H > 0 instead
+      Z1.alloc(nh);
+      Z2.alloc(nh);
+      Z3.alloc(nh);
+    }
     H1.alloc(nh);
-    Z2.alloc(nh);
     H2.alloc(nh);
-    Z3.alloc(nh);
     H3.alloc(nh);
     dH.alloc(nh);
     dZ.alloc(nh);

@@ -129,6 +129,70 @@ __device__ __forceinline__ void store_chunk(const Chunk& ch, int ta, int tb, uin
   }
 }
 
+// acc += A B of one chunk (warp tile 32 x 32 at wm, wn): a fresh MMA accumulator, added to the
+// running sum with compensation
+__device__ __forceinline__ void chunk_product(float (&acc)[2][4][4], float (&cmp)[2][4][4],
+                                              const uint32_t* Ah, const uint32_t* Al,
+                                              const uint32_t* Bh, const uint32_t* Bl, int wm,
+                                              int wn, int gid, int tig) {
+  float part[2][4][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) part[i][j][e] = 0.f;
+#pragma unroll
+  for (int ks = 0; ks < kTK; ks += 8) {
+    uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+      const int r = wm + mt * 16 + gid;
+      ah[mt][0] = Ah[r * kALd + ks + tig];
+      ah[mt][1] = Ah[(r + 8) * kALd + ks + tig];
+      ah[mt][2] = Ah[r * kALd + ks + tig + 4];
+      ah[mt][3] = Ah[(r + 8) * kALd + ks + tig + 4];
+      al[mt][0] = Al[r * kALd + ks + tig];
+      al[mt][1] = Al[(r + 8) * kALd + ks + tig];
+      al[mt][2] = Al[r * kALd + ks + tig + 4];
+      al[mt][3] = Al[(r + 8) * kALd + ks + tig + 4];
+    }
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+      const int cidx = wn + nt * 8 + gid;
+      bh[nt][0] = Bh[(ks + tig) * kBLd + cidx];
+      bh[nt][1] = Bh[(ks + tig + 4) * kBLd + cidx];
+      bl[nt][0] = Bl[(ks + tig) * kBLd + cidx];
+      bl[nt][1] = Bl[(ks + tig + 4) * kBLd + cidx];
+    }
+    // small products first, the chains of the eight tiles interleaved
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int nt = 0; nt < 4; ++nt) mma_tf32(part[mt][nt], al[mt], bh[nt]);
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int nt = 0; nt < 4; ++nt) mma_tf32(part[mt][nt], ah[mt], bl[nt]);
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int nt = 0; nt < 4; ++nt) mma_tf32(part[mt][nt], ah[mt], bh[nt]);
+  }
+  // compensated addition of this chunk's result
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float y = part[i][j][e] - cmp[i][j][e];
+        const float s = acc[i][j][e] + y;
+        cmp[i][j][e] = (s - acc[i][j][e]) - y;
+        acc[i][j][e] = s;
+      }
+}
+
 template <class TA, class TB, class TC>
 __global__ void __launch_bounds__(kThreads, 3)
     k_gemm_tc(const GemmTile* __restrict__ tiles, const GemmTask* __restrict__ tasks,
@@ -178,62 +242,7 @@ __global__ void __launch_bounds__(kThreads, 3)
                          static_cast<const TB*>(b.p[ng.B.base]) + ng.B.off, tl.m0, tl.n0, t.M,
                          t.N, nk0, tid);
     }
-    float part[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) part[i][j][e] = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < kTK; ks += 8) {
-      uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        const int r = wm + mt * 16 + gid;
-        ah[mt][0] = Ah[r * kALd + ks + tig];
-        ah[mt][1] = Ah[(r + 8) * kALd + ks + tig];
-        ah[mt][2] = Ah[r * kALd + ks + tig + 4];
-        ah[mt][3] = Ah[(r + 8) * kALd + ks + tig + 4];
-        al[mt][0] = Al[r * kALd + ks + tig];
-        al[mt][1] = Al[(r + 8) * kALd + ks + tig];
-        al[mt][2] = Al[r * kALd + ks + tig + 4];
-        al[mt][3] = Al[(r + 8) * kALd + ks + tig + 4];
-      }
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        const int cidx = wn + nt * 8 + gid;
-        bh[nt][0] = Bh[(ks + tig) * kBLd + cidx];
-        bh[nt][1] = Bh[(ks + tig + 4) * kBLd + cidx];
-        bl[nt][0] = Bl[(ks + tig) * kBLd + cidx];
-        bl[nt][1] = Bl[(ks + tig + 4) * kBLd + cidx];
-      }
-      // small products first, the chains of the eight tiles interleaved
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) mma_tf32(part[mt][nt], al[mt], bh[nt]);
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) mma_tf32(part[mt][nt], ah[mt], bl[nt]);
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) mma_tf32(part[mt][nt], ah[mt], bh[nt]);
-    }
-    // compensated addition of this chunk's result
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float y = part[i][j][e] - cmp[i][j][e];
-          const float s = acc[i][j][e] + y;
-          cmp[i][j][e] = (s - acc[i][j][e]) - y;
-          acc[i][j][e] = s;
-        }
+    chunk_product(acc, cmp, Ah, Al, Bh, Bl, wm, wn, gid, tig);
     __syncthreads();
     jt = njt;
     k0 = nk0;
@@ -252,6 +261,61 @@ __global__ void __launch_bounds__(kThreads, 3)
           TC* p = C + int64_t(r) * t.C.ld + c;
           *p = beta_zero ? TC(acc[mt][nt][e]) : TC(*p + TC(acc[mt][nt][e]));
         }
+      }
+}
+
+// One dense product C = op(A) op(B) in FP32 storage on the same tiles, its sizes in the launch
+// arguments (no task lists to build, upload and wait for).  blockIdx.z takes the part
+// [z k_len, (z + 1) k_len) of K and writes its own C at z c_split: a 256 x 256 gradient summed
+// over a minibatch has 16 tiles only, and splitting K fills the chip.
+template <DenseEpilogue E>
+__global__ void __launch_bounds__(kThreads, 3) k_dense_tc(const DenseGemm d) {
+  __shared__ __align__(16) uint32_t Ah[kTM * kALd], Al[kTM * kALd];
+  __shared__ __align__(16) uint32_t Bh[kTK * kBLd], Bl[kTK * kBLd];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int gid = lane >> 2, tig = lane & 3;
+  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+  const int m0 = blockIdx.x * kTM, n0 = blockIdx.y * kTN;
+  const int k_beg = blockIdx.z * d.k_len;
+  GemmTerm g{};
+  g.A.ld = d.lda;
+  g.B.ld = d.ldb;
+  g.K = min(d.K, k_beg + d.k_len);
+  g.trans = d.trans;
+  g.alpha = 1.0;
+  float acc[2][4][4], cmp[2][4][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][j][e] = cmp[i][j][e] = 0.f;
+  Chunk ch;
+  if (k_beg < g.K) load_chunk<float, float>(ch, g, d.A, d.B, m0, n0, d.M, d.N, k_beg, tid);
+  for (int k0 = k_beg; k0 < g.K; k0 += kTK) {
+    store_chunk(ch, g.trans & 1, (g.trans >> 1) & 1, Ah, Al, Bh, Bl, tid);
+    __syncthreads();
+    if (k0 + kTK < g.K) load_chunk<float, float>(ch, g, d.A, d.B, m0, n0, d.M, d.N, k0 + kTK, tid);
+    chunk_product(acc, cmp, Ah, Al, Bh, Bl, wm, wn, gid, tig);
+    __syncthreads();
+  }
+  float* C = d.C + int64_t(blockIdx.z) * d.c_split;
+#pragma unroll
+  for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int r = m0 + wm + mt * 16 + gid + (e >= 2 ? 8 : 0);
+        const int c = n0 + wn + nt * 8 + 2 * tig + (e & 1);
+        if (r >= d.M || c >= d.N) continue;
+        float v = acc[mt][nt][e];
+        if (E == DenseEpilogue::bias_relu) {
+          v += d.side[c];
+          v = v > 0.f ? v : 0.f;
+        }
+        if (E == DenseEpilogue::mask) v = d.side[int64_t(r) * d.ldc + c] > 0.f ? v : 0.f;
+        C[int64_t(r) * d.ldc + c] = v;
       }
 }
 
@@ -301,6 +365,19 @@ static void run_gemm_small_mixed(const DevTaskList& L, const Bases<void>& b, int
   const int64_t threads = L.n_small * 32;
   k_gemm_small_f32<TA, TB, TC><<<int((threads + 255) / 256), 256, 0, s>>>(
       L.small_tasks.p, L.n_small, L.terms.p, b, beta_zero, active);
+  DMRG_LAUNCHED();
+}
+
+void dense_gemm_tc(const DenseGemm& d, DenseEpilogue e, int splits, cudaStream_t s) {
+  if (d.M <= 0 || d.N <= 0) return;
+  DMRG_REQUIRE(splits >= 1 && d.k_len >= 1 && int64_t(splits) * d.k_len >= d.K &&
+                   (splits == 1 || e == DenseEpilogue::none),
+               DMRG_EINVAL, "internal: bad split of a dense product");
+  const dim3 grid(unsigned((d.M + kTM - 1) / kTM), unsigned((d.N + kTN - 1) / kTN), unsigned(splits));
+  DMRG_REQUIRE(grid.y <= 65535 && grid.z <= 65535, DMRG_EINVAL, "internal: dense product too large");
+  if (e == DenseEpilogue::none) k_dense_tc<DenseEpilogue::none><<<grid, kThreads, 0, s>>>(d);
+  else if (e == DenseEpilogue::bias_relu) k_dense_tc<DenseEpilogue::bias_relu><<<grid, kThreads, 0, s>>>(d);
+  else k_dense_tc<DenseEpilogue::mask><<<grid, kThreads, 0, s>>>(d);
   DMRG_LAUNCHED();
 }
 
