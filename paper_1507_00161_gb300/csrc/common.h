@@ -84,6 +84,42 @@ struct SectorSet {
 };
 
 // ---------------------------------------------------------------------------------------
+// a second stream for kernels that may run beside others of the main stream: what is launched on
+// it between begin() and end() starts after the main stream's work so far and is complete for
+// the main stream's work after end().  Events only, so it can be captured into a graph.
+// ---------------------------------------------------------------------------------------
+struct SideStream {
+  cudaStream_t s = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  SideStream() = default;
+  SideStream(const SideStream&) = delete;
+  SideStream& operator=(const SideStream&) = delete;
+  ~SideStream() {
+    if (s) {
+      cudaStreamSynchronize(s);
+      cudaStreamDestroy(s);
+    }
+    if (fork) cudaEventDestroy(fork);
+    if (join) cudaEventDestroy(join);
+  }
+  void create() {   // before a capture
+    if (!s) DMRG_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    if (!fork) DMRG_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
+    if (!join) DMRG_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
+  }
+  cudaStream_t begin(cudaStream_t main) {
+    create();
+    DMRG_CUDA(cudaEventRecord(fork, main));
+    DMRG_CUDA(cudaStreamWaitEvent(s, fork, 0));
+    return s;
+  }
+  void end(cudaStream_t main) {
+    DMRG_CUDA(cudaEventRecord(join, s));
+    DMRG_CUDA(cudaStreamWaitEvent(main, join, 0));
+  }
+};
+
+// ---------------------------------------------------------------------------------------
 // device memory: a per-context caching pool.  All device work of a context runs on its one
 // stream, so a block returned to the pool may be handed out again at once (stream order
 // keeps the earlier users ahead).  Blocks are kept in power-of-two classes and released
@@ -478,17 +514,16 @@ struct HeffItem {
 // tile at poff of the scratch, summed later in group order
 struct HeffTile {
   int64_t yoff;
-  int64_t poff;
-  int64_t qoff;               // FP64 tile kernel: four partial tiles (heff.cu)
+  int64_t poff;               // small-block kernel (or -1: written to psi' directly)
+  int64_t qoff;               // tile kernels: four partial tiles, one per slot
   int32_t ld;                 // dRo of the output block
   int32_t r0, c0, m, n;
   int32_t i0, i1;             // items [i0, i1)
   int32_t inst;               // instance (batch mode), 0 for one context
 };
-// deterministic sum of the partial tiles of one output tile: `groups` tiles at poff, or (FP64
-// tile kernel) four per group at qoff.  A list holds the small-block tiles first, then the
-// tile kernels' tiles of several groups, then those of one group (which only the FP64 kernel
-// leaves as partial tiles)
+// deterministic sum of the partial tiles of one output tile: one per group at poff (small-block
+// kernel, grouped passes), or four per group at qoff (tile kernels).  The small-block tiles
+// come first in a superblock's list
 struct HeffRed {
   int64_t yoff, poff, qoff;
   int32_t ld, r0, c0, m, n, groups;
@@ -517,15 +552,22 @@ void heff_small(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_item
                 const HeffPtrs<T>& ptrs, cudaStream_t s);
 template <class T>
 void heff_reduce(const HeffRed* d_red, int64_t n_red, const HeffPtrs<T>& ptrs, cudaStream_t s);
-// mixed path: the same product with 3xTF32 warp MMAs (heff_tc.cu)
-void heff_tc(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
-             const HeffRed* d_red, int64_t n_red, const HeffPtrs<float>& ptrs, cudaStream_t s);
+// sums of the partial tiles of the small-block (the first n_plain entries) and tile kernels
+template <class T>
+void heff_reduce_slots(const HeffRed* d_red, int64_t n_plain, int64_t n_red, const HeffPtrs<T>& ptrs,
+                       cudaStream_t s);
+// mixed path: the same product with 3xTF32 warp MMAs (heff_tc.cu); d_order: the tiles' order by
+// heff_tc_order, whose first n_wide are the wide ones (its return value): wide on s, the
+// narrow ones on s_narrow
+void heff_tc(const HeffTile* d_tiles, const int32_t* d_order, int64_t n_wide, int64_t n_tiles,
+             const HeffItem* d_items, const HeffPtrs<float>& ptrs, cudaStream_t s,
+             cudaStream_t s_narrow);
+int64_t heff_tc_order(const std::vector<HeffTile>& tiles, std::vector<int32_t>& order);
 template <class TO>
 void pad_psi(const double* x, TO* xp, const int64_t* src_off, const int64_t* dst_off,
              const int32_t* len, int nblocks, cudaStream_t s);
-// FP64 tile kernel and its sums (n_plain: small-block entries of the n_red)
+// FP64 tile kernel (its partial tiles are added by heff_reduce_slots)
 void heff_fused64(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
-                  const HeffRed* d_red, int64_t n_plain, int64_t n_red,
                   const HeffPtrs<double>& ptrs, cudaStream_t s);
 // psi into / out of the 16-byte aligned staging copies, with the vector pointers read from
 // device memory (*xp_ptr, *out_ptr) so that a captured graph can be replayed on new vectors

@@ -171,10 +171,11 @@ struct Super {
   DevBuf<HeffItem> fitems;
   DevBuf<HeffTile> ftiles, stiles;   // tile kernels (32 x 32 tiles); small-block kernel
   DevBuf<HeffRed> fred;
-  // sums of partial tiles: small-block tiles, tiles of several groups, of one group (FP64 only)
-  int64_t n_ftiles = 0, n_stiles = 0, n_fred[3] = {0, 0, 0}, p_elems = 0, q_elems = 0;
-  int64_t reds_mixed() const { return n_fred[0] + n_fred[1]; }
-  int64_t reds64() const { return n_fred[0] + n_fred[1] + n_fred[2]; }
+  DevBuf<int32_t> forder;            // order of the tiles in the mixed kernel, n_fwide wide ones first
+  int64_t n_fwide = 0;
+  // sums of partial tiles (n_plain: small-block tiles, first in the list); elements of the
+  // partial tiles of the small-block kernel and of the tile kernels, one after the other
+  int64_t n_ftiles = 0, n_stiles = 0, n_fred = 0, n_plain = 0, p_elems = 0, q_elems = 0;
   std::vector<HeffItem> h_items;
   std::vector<HeffTile> h_tiles, h_stiles;
   std::vector<HeffRed> h_red;
@@ -262,6 +263,7 @@ struct dmrg_ctx {
   int heff_graph = 1;          // replay the product as a CUDA graph (0: eager launches)
   int64_t graph_replays = 0;   // products replayed from a graph
   cudaStream_t cap_stream = nullptr;   // graph capture
+  dmrg::SideStream side;               // kernels of a product that run side by side
   dmrg::DevBuf<float> bigpart32;  // partial blocks of the stage-2 term groups
   dmrg::DevBuf<float> xpad32;
   // precomputed per-site W entry orders (grouped by destination label)
@@ -1076,8 +1078,7 @@ static void build_super(Ctx& c, int p) {
   const int G = 64, Gs = 16;
   std::vector<int64_t> i_beg(nb + 1, 0), t_beg(nb + 1, 0), s_beg(nb + 1, 0), p_beg(nb + 1, 0),
       q_beg(nb + 1, 0), r_beg(nb, 0);
-  int64_t n_red[3] = {0, 0, 0};   // reductions by class: small, several groups, one group
-  std::vector<char> red_class(nb, 0);
+  int64_t n_red[2] = {0, 0};   // sums of partial tiles: small-block tiles, the tile kernels'
   std::vector<char> small_bo(nb, 0), big_bo(nb, 0);
   for (int bo = 0; bo < nb; ++bo) {
     const int ni = int(by_out[bo].size());
@@ -1097,12 +1098,11 @@ static void build_super(Ctx& c, int p) {
     t_beg[bo + 1] = t_beg[bo] + (sm || big ? 0 : tiles * groups);
     s_beg[bo + 1] = s_beg[bo] + (sm ? groups : 0);
     if (!big && !(sm && groups == 1)) {
-      red_class[bo] = sm ? 0 : groups > 1 ? 1 : 2;
-      r_beg[bo] = n_red[int(red_class[bo])];
-      n_red[int(red_class[bo])] += tiles;
+      r_beg[bo] = n_red[sm ? 0 : 1];
+      n_red[sm ? 0 : 1] += tiles;
     }
     q_beg[bo + 1] = q_beg[bo] + (sm || big ? 0 : int64_t(4) * groups * sb->bdl[bo] * sb->bdr[bo]);
-    p_beg[bo + 1] = p_beg[bo] + (groups > 1 && !big ? int64_t(groups) * sb->bdl[bo] * sb->bdr[bo] : 0);
+    p_beg[bo + 1] = p_beg[bo] + (groups > 1 && sm ? int64_t(groups) * sb->bdl[bo] * sb->bdr[bo] : 0);
   }
   DMRG_REQUIRE(i_beg[nb] < (int64_t(1) << 31), DMRG_EINVAL, "superblock has too many terms");
   struct TileCost {
@@ -1111,11 +1111,9 @@ static void build_super(Ctx& c, int p) {
   };
   std::vector<HeffItem> fi(i_beg[nb]);
   std::vector<TileCost> ft(t_beg[nb]), fts(s_beg[nb]);
-  std::vector<HeffRed> fr(n_red[0] + n_red[1] + n_red[2]);
-  for (int bo = 0; bo < nb; ++bo) {
-    if (red_class[bo] > 0) r_beg[bo] += n_red[0];
-    if (red_class[bo] > 1) r_beg[bo] += n_red[1];
-  }
+  std::vector<HeffRed> fr(n_red[0] + n_red[1]);
+  for (int bo = 0; bo < nb; ++bo)
+    if (!small_bo[bo]) r_beg[bo] += n_red[0];
   std::vector<double> bo_flops(nb, 0.0), bo_bytes(nb, 0.0), bo_kflops(nb, 0.0);
   std::vector<int64_t> bo_toff(nb, 0);
   std::vector<std::array<double, 8>> bo_hist(nb);
@@ -1194,11 +1192,11 @@ static void build_super(Ctx& c, int p) {
           for (int g = 0; g < groups; ++g) {
             t.i0 = i0 + g * GG;
             t.i1 = std::min(i1, t.i0 + GG);
-            t.poff = groups > 1 ? pelems + g * mn : -1;
+            t.poff = sm && groups > 1 ? pelems + g * mn : -1;
             t.qoff = sm ? 0 : qelems + 4 * g * mn;
             dst[tpos++] = TileCost{t, work * double(t.i1 - t.i0) / std::max(1, i1 - i0) * t.n + 1.0};
           }
-          if (groups > 1) pelems += groups * mn;
+          if (sm && groups > 1) pelems += groups * mn;
           if (!sm) qelems += 4 * groups * mn;
         }
     }
@@ -1256,12 +1254,16 @@ static void build_super(Ctx& c, int p) {
     check(ft, tl, 32);
     check(fts, tls, kSmallEdge);
     for (const HeffRed& r : fr)
-      DMRG_REQUIRE((r.groups == 1 || r.poff + int64_t(r.groups) * r.m * r.n <= pelems) &&
-                       r.qoff + (r.qoff ? int64_t(4) * r.groups * r.m * r.n : 0) <= qend &&
+      DMRG_REQUIRE((&r - fr.data() < n_red[0]
+                        ? r.poff + int64_t(r.groups) * r.m * r.n <= pelems
+                        : r.qoff + int64_t(4) * r.groups * r.m * r.n <= qend) &&
                        r.yoff + int64_t(r.r0 + r.m - 1) * r.ld + r.c0 + r.n - 1 < sb->size,
                    DMRG_EINVAL, "internal: partial tile out of range");
     sb->fitems.upload(fi, c.stream);
     sb->ftiles.upload(tl, c.stream);
+    std::vector<int32_t> order;
+    sb->n_fwide = heff_tc_order(tl, order);
+    sb->forder.upload(order, c.stream);
     sb->stiles.upload(tls, c.stream);
     sb->fred.upload(fr, c.stream);
     // host copies for batch mode (lists of several instances in one launch)
@@ -1275,7 +1277,8 @@ static void build_super(Ctx& c, int p) {
     for (size_t i = 0; i < fts.size(); ++i) sb->h_scost[i] = fts[i].cost;
     sb->n_ftiles = int64_t(sb->h_tiles.size());
     sb->n_stiles = int64_t(sb->h_stiles.size());
-    std::copy(n_red, n_red + 3, sb->n_fred);
+    sb->n_fred = int64_t(sb->h_red.size());
+    sb->n_plain = n_red[0];
     sb->p_elems = pelems;
     sb->q_elems = q_beg[nb];
   }
@@ -1466,7 +1469,7 @@ static void heff_buffers(Ctx& c, Super& sb, int prec) {
     }
   } else {
     c.f32b.alloc(std::max<int64_t>(sb.size, 1));
-    c.part32.alloc(std::max<int64_t>(sb.p_elems, 1));
+    c.part32.alloc(std::max<int64_t>(sb.p_elems + sb.q_elems, 1));
     c.xpad32.alloc(sb.pad_size);
     if (sb.n_big_blocks) {
       c.f32T.alloc(std::max<int64_t>(sb.big_t_elems, 1));
@@ -1475,12 +1478,82 @@ static void heff_buffers(Ctx& c, Super& sb, int prec) {
   }
 }
 
-// the product's kernels after the staging of psi: small blocks, fused tiles, grouped passes
-// of the big output blocks and their reductions.  FP64 writes psi' to y64; the mixed path to
-// the FP32 buffer c.f32b.  Every psi' element is written by exactly one fused tile or one
+// The kernels of the output blocks of one precision on main stream st: small blocks, tiles, and
+// the two grouped passes of the big blocks (`big`, writing to their own blocks).  They do not
+// depend on each other, and each alone leaves the chip partly idle (its last wave; a few large
+// tasks), so they run side by side: the grouped passes, or else the wide tiles, on st, the rest
+// on the side stream; then the partial tiles are added.  Measured (GB300): pf 4p+4n at
+// position 6 (five short kernels) 136 -> 89 us per product, the mixed one of pf 4p+5n 83 -> 78 us.
+struct TileLists {
+  const HeffTile *stiles, *tiles;
+  const int32_t* order;
+  const HeffItem* items;
+  const HeffRed* red;
+  int64_t n_stiles, n_tiles, n_wide, n_plain, n_red;
+};
+template <class F>
+static void tile_kernels(const TileLists& l, const HeffPtrs<double>& p, SideStream& side,
+                         cudaStream_t st, bool any_big, F&& big) {
+  cudaStream_t sd = side.begin(st);
+  heff_small<double>(l.stiles, l.n_stiles, l.items, p, sd);
+  heff_fused64(l.tiles, l.n_tiles, l.items, p, any_big ? sd : st);
+  if (any_big) big();
+  side.end(st);
+  heff_reduce_slots<double>(l.red, l.n_plain, l.n_red, p, st);
+}
+template <class F>
+static void tile_kernels(const TileLists& l, const HeffPtrs<float>& p, SideStream& side,
+                         cudaStream_t st, bool any_big, F&& big) {
+  cudaStream_t sd = side.begin(st);
+  heff_small<float>(l.stiles, l.n_stiles, l.items, p, sd);
+  heff_tc(l.tiles, l.order, l.n_wide, l.n_tiles, l.items, p, any_big ? sd : st, sd);
+  if (any_big) big();
+  side.end(st);
+  heff_reduce_slots<float>(l.red, l.n_plain, l.n_red, p, st);
+}
+
+// grouped GEMM passes of one superblock's big output blocks
+static void big_passes(Ctx& c, Super& sb, double* y, const int32_t* active, cudaStream_t st) {
+  Bases<double> bb{};
+  bb.p[B_LOPS] = sb.L.data.p;
+  bb.p[B_ROPS] = sb.R.data.p;
+  bb.p[B_X] = c.xpad64.p;
+  bb.p[B_Y] = y;
+  bb.p[B_T] = c.T.p;
+  bb.p[B_Z] = c.bigpart64.p;
+  run_gemm_tasks<double>(sb.big1, bb, 1, st, active);
+  run_gemm_tasks<double>(sb.big2, bb, 1, st, active);
+  HeffPtrs<double> rp{};
+  rp.Y[0] = y;
+  rp.P[0] = c.bigpart64.p;
+  rp.active = active;
+  heff_reduce<double>(sb.big_red.p, sb.n_big_red, rp, st);
+}
+static void big_passes(Ctx& c, Super& sb, float* y, const int32_t* active, cudaStream_t st) {
+  Bases<void> bb{};
+  bb.p[B_LOPS] = sb.L.data32.p;
+  bb.p[B_ROPS] = sb.R.data32.p;
+  bb.p[B_X] = c.xpad32.p;
+  bb.p[B_Y] = y;
+  bb.p[B_T] = c.f32T.p;
+  bb.p[B_Z] = c.bigpart32.p;
+  run_gemm_tasks_tc<float, float, float>(sb.big1, bb, 1, st, active);
+  run_gemm_tasks_tc<float, float, float>(sb.big2, bb, 1, st, active);
+  HeffPtrs<float> rp{};
+  rp.Y[0] = y;
+  rp.P[0] = c.bigpart32.p;
+  rp.active = active;
+  heff_reduce<float>(sb.big_red.p, sb.n_big_red, rp, st);
+}
+
+// the product's kernels after the staging of psi.  FP64 writes psi' to y64; the mixed path to
+// the FP32 buffer c.f32b.  Every psi' element is written by exactly one tile or one
 // grouped-GEMM task (blocks without terms get zero-term tiles or tasks), so no clearing pass
 // is needed.
 static void heff_core(Ctx& c, Super& sb, int prec, double* y64, cudaStream_t st) {
+  const TileLists l{sb.stiles.p, sb.ftiles.p, sb.forder.p, sb.fitems.p, sb.fred.p, sb.n_stiles,
+                    sb.n_ftiles, sb.n_fwide, sb.n_plain, sb.n_fred};
+  const bool big = sb.n_big_blocks > 0;
   if (prec == 0) {
     HeffPtrs<double> ptr{};
     ptr.L[0] = sb.L.data.p;
@@ -1488,24 +1561,7 @@ static void heff_core(Ctx& c, Super& sb, int prec, double* y64, cudaStream_t st)
     ptr.X[0] = c.xpad64.p;
     ptr.Y[0] = y64;
     ptr.P[0] = c.part64.p;
-    heff_small<double>(sb.stiles.p, sb.n_stiles, sb.fitems.p, ptr, st);
-    heff_fused64(sb.ftiles.p, sb.n_ftiles, sb.fitems.p, sb.fred.p, sb.n_fred[0], sb.reds64(), ptr,
-                 st);
-    if (sb.n_big_blocks) {
-      Bases<double> bb{};
-      bb.p[B_LOPS] = sb.L.data.p;
-      bb.p[B_ROPS] = sb.R.data.p;
-      bb.p[B_X] = c.xpad64.p;
-      bb.p[B_Y] = y64;
-      bb.p[B_T] = c.T.p;
-      bb.p[B_Z] = c.bigpart64.p;
-      run_gemm_tasks<double>(sb.big1, bb, 1, st);
-      run_gemm_tasks<double>(sb.big2, bb, 1, st);
-      HeffPtrs<double> rp{};
-      rp.Y[0] = y64;
-      rp.P[0] = c.bigpart64.p;
-      heff_reduce<double>(sb.big_red.p, sb.n_big_red, rp, st);
-    }
+    tile_kernels(l, ptr, c.side, st, big, [&] { big_passes(c, sb, y64, nullptr, st); });
   } else {
     HeffPtrs<float> ptr{};
     ptr.L[0] = sb.L.data32.p;
@@ -1513,23 +1569,7 @@ static void heff_core(Ctx& c, Super& sb, int prec, double* y64, cudaStream_t st)
     ptr.X[0] = c.xpad32.p;
     ptr.Y[0] = c.f32b.p;
     ptr.P[0] = c.part32.p;
-    heff_small<float>(sb.stiles.p, sb.n_stiles, sb.fitems.p, ptr, st);
-    heff_tc(sb.ftiles.p, sb.n_ftiles, sb.fitems.p, sb.fred.p, sb.reds_mixed(), ptr, st);
-    if (sb.n_big_blocks) {
-      Bases<void> bb{};
-      bb.p[B_LOPS] = sb.L.data32.p;
-      bb.p[B_ROPS] = sb.R.data32.p;
-      bb.p[B_X] = c.xpad32.p;
-      bb.p[B_Y] = c.f32b.p;
-      bb.p[B_T] = c.f32T.p;
-      bb.p[B_Z] = c.bigpart32.p;
-      run_gemm_tasks_tc<float, float, float>(sb.big1, bb, 1, st);
-      run_gemm_tasks_tc<float, float, float>(sb.big2, bb, 1, st);
-      HeffPtrs<float> rp{};
-      rp.Y[0] = c.f32b.p;
-      rp.P[0] = c.bigpart32.p;
-      heff_reduce<float>(sb.big_red.p, sb.n_big_red, rp, st);
-    }
+    tile_kernels(l, ptr, c.side, st, big, [&] { big_passes(c, sb, c.f32b.p, nullptr, st); });
   }
 }
 
@@ -1550,6 +1590,7 @@ static void heff_graph_key(const Ctx& c, int prec, const void* (&k)[6]) {
 static void heff_capture(Ctx& c, Super& sb, int prec) {
   Super::Graph& G = sb.graph[prec];
   if (!c.cap_stream) DMRG_CUDA(cudaStreamCreateWithFlags(&c.cap_stream, cudaStreamNonBlocking));
+  c.side.create();
   cudaGraph_t g = nullptr;
   DMRG_CUDA(cudaStreamBeginCapture(c.cap_stream, cudaStreamCaptureModeThreadLocal));
   try {
@@ -3801,13 +3842,16 @@ struct dmrg_batch {
   std::vector<dmrg_ctx*> ctx;
   int precision = DMRG_FP64;
   cudaStream_t bs = nullptr;                 // internal stream (graph capture)
+  dmrg::SideStream side;
   cudaEvent_t ev = nullptr;
   std::vector<cudaEvent_t> ev_ctx;
   // combined lists of the current step
   dmrg::DevBuf<dmrg::HeffItem> items;
   dmrg::DevBuf<dmrg::HeffTile> tiles, stiles;
   dmrg::DevBuf<dmrg::HeffRed> red;
-  int64_t n_tiles = 0, n_stiles = 0, n_red[3] = {0, 0, 0};   // (reductions by class, see Super)
+  dmrg::DevBuf<int32_t> order;
+  int64_t n_wide = 0;
+  int64_t n_tiles = 0, n_stiles = 0, n_red = 0, n_plain = 0;
   // per-iteration tables: input and output vector pointers, active flags
   struct Tab {
     const double* in[dmrg::kMaxInst];
@@ -3846,7 +3890,7 @@ struct PoolScope {
 static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
   std::vector<HeffItem> fi;
   std::vector<std::pair<double, HeffTile>> ft, fts;
-  std::vector<HeffRed> fr[3];
+  std::vector<HeffRed> fr, fr_tiles;   // small-block tiles first
   for (int i : inst) {
     Super& sb = *B.ctx[i]->sb;
     const int base = int(fi.size());
@@ -3863,13 +3907,11 @@ static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
     };
     add(sb.h_tiles, sb.h_cost, ft);
     add(sb.h_stiles, sb.h_scost, fts);
-    size_t at = 0;
-    for (int k = 0; k < 3; ++k)
-      for (int64_t x = 0; x < sb.n_fred[k]; ++x) {
-        HeffRed r = sb.h_red[at++];
-        r.inst = i;
-        fr[k].push_back(r);
-      }
+    for (size_t x = 0; x < sb.h_red.size(); ++x) {
+      HeffRed r = sb.h_red[x];
+      r.inst = i;
+      (int64_t(x) < sb.n_plain ? fr : fr_tiles).push_back(r);
+    }
   }
   auto sorted = [](std::vector<std::pair<double, HeffTile>>& v) {
     std::stable_sort(v.begin(), v.end(),
@@ -3881,12 +3923,14 @@ static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
   const std::vector<HeffTile> tl = sorted(ft), tls = sorted(fts);
   B.items.upload(fi, B.bs);
   B.tiles.upload(tl, B.bs);
+  std::vector<int32_t> order;
+  B.n_wide = heff_tc_order(tl, order);
+  B.order.upload(order, B.bs);
   B.stiles.upload(tls, B.bs);
-  for (int k = 0; k < 3; ++k) {
-    B.n_red[k] = int64_t(fr[k].size());
-    if (k) fr[0].insert(fr[0].end(), fr[k].begin(), fr[k].end());
-  }
-  B.red.upload(fr[0], B.bs);
+  B.n_plain = int64_t(fr.size());
+  fr.insert(fr.end(), fr_tiles.begin(), fr_tiles.end());
+  B.n_red = int64_t(fr.size());
+  B.red.upload(fr, B.bs);
   B.n_tiles = int64_t(tl.size());
   B.n_stiles = int64_t(tls.size());
   DMRG_CUDA(cudaStreamSynchronize(B.bs));
@@ -3896,6 +3940,10 @@ static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
 // instance into its staging copy, one fused launch, one reduction, results out
 static void batch_issue(dmrg_batch& B, const std::vector<int>& inst) {
   const int32_t* act = B.d_tab->active;
+  const TileLists l{B.stiles.p, B.tiles.p, B.order.p, B.items.p, B.red.p, B.n_stiles,
+                    B.n_tiles, B.n_wide, B.n_plain, B.n_red};
+  bool any_big = false;
+  for (int i : inst) any_big = any_big || B.ctx[i]->sb->n_big_blocks > 0;
   if (B.precision == DMRG_FP64) {
     HeffPtrs<double> ptr{};
     ptr.active = act;
@@ -3910,28 +3958,12 @@ static void batch_issue(dmrg_batch& B, const std::vector<int>& inst) {
       ptr.Y[i] = c.ybat64.p;
       ptr.P[i] = c.part64.p;
     }
-    heff_small<double>(B.stiles.p, B.n_stiles, B.items.p, ptr, B.bs);
-    heff_fused64(B.tiles.p, B.n_tiles, B.items.p, B.red.p, B.n_red[0],
-                 B.n_red[0] + B.n_red[1] + B.n_red[2], ptr, B.bs);
-    for (int i : inst) {   // big output blocks: grouped GEMM passes per instance
-      Ctx& c = *B.ctx[i];
-      Super& sb = *c.sb;
-      if (!sb.n_big_blocks) continue;
-      Bases<double> bb{};
-      bb.p[B_LOPS] = sb.L.data.p;
-      bb.p[B_ROPS] = sb.R.data.p;
-      bb.p[B_X] = c.xpad64.p;
-      bb.p[B_Y] = c.ybat64.p;
-      bb.p[B_T] = c.T.p;
-      bb.p[B_Z] = c.bigpart64.p;
-      run_gemm_tasks<double>(sb.big1, bb, 1, B.bs, act + i);
-      run_gemm_tasks<double>(sb.big2, bb, 1, B.bs, act + i);
-      HeffPtrs<double> rp{};
-      rp.Y[0] = c.ybat64.p;
-      rp.P[0] = c.bigpart64.p;
-      rp.active = act + i;
-      heff_reduce<double>(sb.big_red.p, sb.n_big_red, rp, B.bs);
-    }
+    tile_kernels(l, ptr, B.side, B.bs, any_big, [&] {   // grouped passes per instance
+      for (int i : inst) {
+        Ctx& c = *B.ctx[i];
+        if (c.sb->n_big_blocks) big_passes(c, *c.sb, c.ybat64.p, act + i, B.bs);
+      }
+    });
     for (int i : inst) {
       Ctx& c = *B.ctx[i];
       out_to_f64_ind<double>(c.ybat64.p, &B.d_tab->out[i], c.sb->size, act + i, B.bs);
@@ -3950,27 +3982,12 @@ static void batch_issue(dmrg_batch& B, const std::vector<int>& inst) {
       ptr.Y[i] = c.f32b.p;
       ptr.P[i] = c.part32.p;
     }
-    heff_small<float>(B.stiles.p, B.n_stiles, B.items.p, ptr, B.bs);
-    heff_tc(B.tiles.p, B.n_tiles, B.items.p, B.red.p, B.n_red[0] + B.n_red[1], ptr, B.bs);
-    for (int i : inst) {   // big output blocks: grouped GEMM passes per instance
-      Ctx& c = *B.ctx[i];
-      Super& sb = *c.sb;
-      if (!sb.n_big_blocks) continue;
-      Bases<void> bb{};
-      bb.p[B_LOPS] = sb.L.data32.p;
-      bb.p[B_ROPS] = sb.R.data32.p;
-      bb.p[B_X] = c.xpad32.p;
-      bb.p[B_Y] = c.f32b.p;
-      bb.p[B_T] = c.f32T.p;
-      bb.p[B_Z] = c.bigpart32.p;
-      run_gemm_tasks_tc<float, float, float>(sb.big1, bb, 1, B.bs, act + i);
-      run_gemm_tasks_tc<float, float, float>(sb.big2, bb, 1, B.bs, act + i);
-      HeffPtrs<float> rp{};
-      rp.Y[0] = c.f32b.p;
-      rp.P[0] = c.bigpart32.p;
-      rp.active = act + i;
-      heff_reduce<float>(sb.big_red.p, sb.n_big_red, rp, B.bs);
-    }
+    tile_kernels(l, ptr, B.side, B.bs, any_big, [&] {
+      for (int i : inst) {
+        Ctx& c = *B.ctx[i];
+        if (c.sb->n_big_blocks) big_passes(c, *c.sb, c.f32b.p, act + i, B.bs);
+      }
+    });
     for (int i : inst) {
       Ctx& c = *B.ctx[i];
       out_to_f64_ind<float>(c.f32b.p, &B.d_tab->out[i], c.sb->size, act + i, B.bs);
@@ -3994,7 +4011,7 @@ static void batch_buffers(dmrg_batch& B, const std::vector<int>& inst) {
       }
     } else {
       c.f32b.alloc(std::max<int64_t>(sb.size, 1));
-      c.part32.alloc(std::max<int64_t>(sb.p_elems, 1));
+      c.part32.alloc(std::max<int64_t>(sb.p_elems + sb.q_elems, 1));
       c.xpad32.alloc(sb.pad_size);
       if (sb.n_big_blocks) {
         c.f32T.alloc(std::max<int64_t>(sb.big_t_elems, 1));
@@ -4158,6 +4175,7 @@ extern "C" int dmrg_batch_create(int32_t n, dmrg_ctx* const* ctxs, dmrg_batch** 
     }
     b->precision = ctxs[0]->opt.precision;
     DMRG_CUDA(cudaStreamCreateWithFlags(&b->bs, cudaStreamNonBlocking));
+    b->side.create();
     DMRG_CUDA(cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming));
     b->ev_ctx.resize(n);
     for (int i = 0; i < n; ++i) DMRG_CUDA(cudaEventCreateWithFlags(&b->ev_ctx[i], cudaEventDisableTiming));

@@ -146,22 +146,24 @@ k_heff_fused(const HeffTile* __restrict__ tiles, const HeffItem* __restrict__ it
 // psi' tile = sum over groups (in group order) of the partial tiles, each the sum of its slots
 // in order: red[0 .. n_plain) have one partial tile per group (poff; the small-block kernel),
 // the others four (qoff)
+template <class T>
 __global__ void __launch_bounds__(128)
-k_heff_reduce_slots(const HeffRed* __restrict__ red, int64_t n_plain, const HeffPtrs<double> ptrs) {
+k_heff_reduce_slots(const HeffRed* __restrict__ red, int64_t n_plain, const HeffPtrs<T> ptrs) {
   const HeffRed r = red[blockIdx.x];
   if (ptrs.active && !ptrs.active[r.inst]) return;
   const bool plain = blockIdx.x < n_plain;
-  const double* __restrict__ P = ptrs.P[r.inst] + (plain ? r.poff : r.qoff);
-  double* __restrict__ Y = ptrs.Y[r.inst];
+  const T* __restrict__ P = ptrs.P[r.inst] + (plain ? r.poff : r.qoff);
+  T* __restrict__ Y = ptrs.Y[r.inst];
   const int mn = r.m * r.n;
   for (int e = threadIdx.x; e < mn; e += blockDim.x) {
-    double s = 0.0;
+    T s = T(0);
+#pragma unroll 4
     for (int g = 0; g < r.groups; ++g) {
       if (plain) {
         s += P[int64_t(g) * mn + e];
       } else {
-        const double* q = P + int64_t(g) * kSlots * mn + e;
-        double u = q[0];
+        const T* q = P + int64_t(g) * kSlots * mn + e;
+        T u = q[0];
 #pragma unroll
         for (int w = 1; w < kSlots; ++w) u += q[int64_t(w) * mn];
         s = r.groups > 1 ? s + u : u;
@@ -210,17 +212,23 @@ void heff_reduce(const HeffRed* d_red, int64_t n_red, const HeffPtrs<T>& ptrs, c
 template void heff_reduce<float>(const HeffRed*, int64_t, const HeffPtrs<float>&, cudaStream_t);
 template void heff_reduce<double>(const HeffRed*, int64_t, const HeffPtrs<double>&, cudaStream_t);
 
+template <class T>
+void heff_reduce_slots(const HeffRed* d_red, int64_t n_plain, int64_t n_red, const HeffPtrs<T>& ptrs,
+                       cudaStream_t s) {
+  if (n_red <= 0) return;
+  k_heff_reduce_slots<T><<<int(n_red), 128, 0, s>>>(d_red, n_plain, ptrs);
+  DMRG_LAUNCHED();
+}
+template void heff_reduce_slots<float>(const HeffRed*, int64_t, int64_t, const HeffPtrs<float>&,
+                                       cudaStream_t);
+template void heff_reduce_slots<double>(const HeffRed*, int64_t, int64_t, const HeffPtrs<double>&,
+                                        cudaStream_t);
+
 void heff_fused64(const HeffTile* d_tiles, int64_t n_tiles, const HeffItem* d_items,
-                  const HeffRed* d_red, int64_t n_plain, int64_t n_red,
                   const HeffPtrs<double>& ptrs, cudaStream_t s) {
-  if (n_tiles > 0) {
-    k_heff_fused<<<int(n_tiles * kSlots), kThr, 0, s>>>(d_tiles, d_items, ptrs);
-    DMRG_LAUNCHED();
-  }
-  if (n_red > 0) {
-    k_heff_reduce_slots<<<int(n_red), 128, 0, s>>>(d_red, n_plain, ptrs);
-    DMRG_LAUNCHED();
-  }
+  if (n_tiles <= 0) return;
+  k_heff_fused<<<int(n_tiles * kSlots), kThr, 0, s>>>(d_tiles, d_items, ptrs);
+  DMRG_LAUNCHED();
 }
 
 // staging with the vector pointer read from device memory (graph replay on new vectors)
