@@ -254,12 +254,14 @@ k_dav_next(const double* __restrict__ t, const double* __restrict__ tt,
 // the time is the count of FP64 instructions on the critical path.  A rotation takes 30 of them
 // here against 47 with library divisions and roots, comparisons included; a round rotates the
 // matrix in 4.
-//   - Warp 0 forms the rotations.  Signs, zeros and powers of two are handled as integers.
-//   - The other warps meanwhile rotate V with the previous round's angles, and before the first
-//     round of a sweep sum the off-diagonal norm; V is only needed at the end.
+//   - Warp 0 forms the rotations of the next round while the other warps apply this round's to A
+//     and V: it first rotates the three elements per pair that it needs itself (A is double-
+//     buffered), so the chain of divisions and roots never waits for the matrix.  Signs, zeros
+//     and powers of two are handled as integers.
 //   - Rows and columns of A are rotated in one pass, four lanes per 2 x 2 block (the rows of one
 //     pair, the columns of another): one element each, exchanged by shuffles.
-// Measured (GB300): 4400 clocks per round against 5700; a problem of 8 vectors 77 us, of 16 190 us.
+// Measured (GB300) against rotations, rows, columns one after the other with library divisions:
+// 3900 clocks per round against 5700; 8 vectors 65 us, 16 vectors 170 us, 24 vectors 340 us.
 // ------------------------------------------------------------------------------------
 constexpr int kMaxK = 64;
 
@@ -347,115 +349,208 @@ __device__ __forceinline__ void pair_of(int m, int r, int a, int& p, int& q) {
 struct RitzShared {
   double c[2][kMaxK / 2], s[2][kMaxK / 2];   // rotations, double-buffered by round
   int p[2][kMaxK / 2], q[2][kMaxK / 2];
-  double off[kWarps], tot[kWarps], w[kMaxK];
+  double norm[2 * kWarps], w[kMaxK];   // off-diagonal and whole norm by warp
   int low[2];
+  // pair a of round r at [r * half + a]: p, q, and of each its partner and its pair's number in
+  // the round before (6 bits each)
+  uint32_t low_bits[(kMaxK - 1) * kMaxK / 2], high_bits[(kMaxK - 1) * kMaxK / 2];
 };
+struct PairOf {
+  int p, q, p_mate, q_mate, p_pair, q_pair;
+};
+__device__ __forceinline__ PairOf pair_entry(const RitzShared& sh, int at) {
+  const uint32_t l = sh.low_bits[at], h = sh.high_bits[at];
+  return {int(l & 63), int(l >> 6 & 63), int(l >> 12 & 63), int(l >> 18 & 63), int(h & 63),
+          int(h >> 6 & 63)};
+}
 
-// columns of V by the rotations of buffer `buf`, by the threads first, first + step, ...
-__device__ __forceinline__ void rotate_v(double* V, int k, int half, const RitzShared& sh, int buf,
-                                         int first, int step) {
-  for (int e = first; e < half * k; e += step) {
-    const int a = e / k, row = e - a * k;
-    const int p = sh.p[buf][a], q = sh.q[buf][a];
-    const double c = sh.c[buf][a], s = sh.s[buf][a];
-    if (q >= k || is_zero(s)) continue;
-    const double vp = V[row * k + p], vq = V[row * k + q];
-    V[row * k + p] = fma(c, vp, -(s * vq));
-    V[row * k + q] = fma(s, vp, c * vq);
+// x_p, x_q -> c x_p - s x_q, s x_p + c x_q (first product fused, second rounded)
+__device__ __forceinline__ double rotated(double xp, double xq, double c, double s, bool is_q) {
+  return fma(is_q ? s : c, xp, flip_if((is_q ? c : s) * xq, !is_q));
+}
+
+// element (i, j) of A (k x k) after the rotations of buffer buf: i was paired with i_mate in pair
+// i_pair, j likewise
+__device__ __forceinline__ double element_after(const double* A, int k, const RitzShared& sh, int buf,
+                                                int i, int i_mate, int i_pair, int j, int j_mate,
+                                                int j_pair) {
+  const double ca = sh.c[buf][i_pair], sa = sh.s[buf][i_pair];
+  const double cb = sh.c[buf][j_pair], sb = sh.s[buf][j_pair];
+  const int i2 = min(i_mate, k - 1), j2 = min(j_mate, k - 1);   // (a bye has no rotation)
+  const double x_ij = A[i * k + j], x_2j = A[i2 * k + j], x_i2 = A[i * k + j2], x_22 = A[i2 * k + j2];
+  const bool lo = i > i_mate, right = j > j_mate;
+  double y = x_ij, y2 = x_i2;
+  if (!is_zero(sa)) {
+    y = rotated(lo ? x_2j : x_ij, lo ? x_ij : x_2j, ca, sa, lo);
+    y2 = rotated(lo ? x_22 : x_i2, lo ? x_i2 : x_22, ca, sa, lo);
+  }
+  return is_zero(sb) ? y : rotated(right ? y2 : y, right ? y : y2, cb, sb, right);
+}
+
+// rotations of round r into buffer buf (one warp): the elements read from A, or (after) as they
+// will be once the rotations of buffer buf ^ 1 (the round before) have been applied to A
+__device__ __forceinline__ void round_rotations(const double* A, int k, int half, int r, bool after,
+                                                RitzShared& sh, int buf) {
+  const int lane = threadIdx.x & 31;
+  // lane -> pair a, and which of its elements (p, p), (q, q), (p, q) the lane rotates first
+  int g = 0, a = lane;
+  if (3 * half <= 32) {
+    g = lane >= 2 * half ? 2 : lane >= half ? 1 : 0;
+    a = lane - g * half;
+  } else if (half <= 16) {
+    g = lane >> 4;
+    a = lane & 15;
+  }
+  const PairOf e = pair_entry(sh, r * half + min(a, half - 1));
+  const int p = e.p, q = e.q;
+  const bool bye = q >= k;
+  double app, aqq = 0.0, apq = 0.0;
+  if (!after) {
+    app = A[p * k + p];
+    if (!bye) {
+      aqq = A[q * k + q];
+      apq = A[p * k + q];
+    }
+  } else if (3 * half <= 32) {   // the three elements of all pairs at once
+    const bool iq = g == 1, jq = g > 0;   // (p, p), (q, q), (p, q)
+    const double x =
+        bye && g > 0 ? 0.0
+                     : element_after(A, k, sh, buf ^ 1, iq ? q : p, iq ? e.q_mate : e.p_mate,
+                                     iq ? e.q_pair : e.p_pair, jq ? q : p, jq ? e.q_mate : e.p_mate,
+                                     jq ? e.q_pair : e.p_pair);
+    app = x;
+    aqq = __shfl_sync(0xffffffffu, x, (lane + half) & 31);
+    apq = __shfl_sync(0xffffffffu, x, (lane + 2 * half) & 31);
+  } else {
+    const bool is_q = g == 1;
+    app = is_q && bye ? 0.0
+                      : element_after(A, k, sh, buf ^ 1, is_q ? q : p, is_q ? e.q_mate : e.p_mate,
+                                      is_q ? e.q_pair : e.p_pair, is_q ? q : p,
+                                      is_q ? e.q_mate : e.p_mate, is_q ? e.q_pair : e.p_pair);
+    if (half <= 16)
+      aqq = __shfl_sync(0xffffffffu, app, (lane + 16) & 31);
+    else if (!bye)
+      aqq = element_after(A, k, sh, buf ^ 1, q, e.q_mate, e.q_pair, q, e.q_mate, e.q_pair);
+    if (!bye) apq = element_after(A, k, sh, buf ^ 1, p, e.p_mate, e.p_pair, q, e.q_mate, e.q_pair);
+  }
+  if (lane >= half || bye) apq = 0.0;   // (spare lanes and a bye: no rotation)
+  double c, s;
+  rotation(0xffffffffu, app, aqq, apq, c, s);
+  if (lane < half) {
+    sh.p[buf][lane] = p;
+    sh.q[buf][lane] = q;
+    sh.c[buf][lane] = c;
+    sh.s[buf][lane] = s;
   }
 }
 
 __device__ void ritz_block(const double* H, int ld, int k, double* sm, double* w, double* Y) {
   __shared__ RitzShared sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  double* A = sm;
-  double* V = sm + k * k;
+  double* A = sm;              // before a round
+  double* B = sm + k * k;      // after it
+  double* V = sm + 2 * k * k;
+  double off = 0.0, tot = 0.0;   // off-diagonal Frobenius norm against the full norm
+  auto norms = [&](double x, bool diagonal) {
+    tot = fma(x, x, tot);
+    if (!diagonal) off = fma(x, x, off);
+  };
+  auto norms_out = [&] {   // lanes 0-15 add the one, 16-31 the other
+    const bool up = lane & 16;
+    double x = (up ? tot : off) + __shfl_xor_sync(0xffffffffu, up ? off : tot, 16);
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((lane & 15) == 0) sh.norm[(up ? kWarps : 0) + warp] = x;
+    off = tot = 0.0;
+  };
+  auto converged = [&] {   // the same sums in every warp
+    double x = sh.norm[lane & 15];
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    const double o = __shfl_sync(0xffffffffu, x, 0), t = __shfl_sync(0xffffffffu, x, 8);
+    return o <= 1e-30 * t || t == 0.0;
+  };
   for (int i = tid; i < k * k; i += kThr) {
     const int r = i / k, c = i - r * k;
-    A[i] = (r >= c) ? __ldcg(H + r * ld + c) : __ldcg(H + c * ld + r);
+    const double x = (r >= c) ? __ldcg(H + r * ld + c) : __ldcg(H + c * ld + r);
+    A[i] = x;
     V[i] = r == c ? 1.0 : 0.0;
+    norms(x, r == c);
+  }
+  norms_out();
+  const int m = (k + 1) & ~1, half = m / 2;
+  for (int i = tid; i < (m - 1) * half; i += kThr) {
+    const int r = i / half;
+    int p, q;
+    pair_of(m, r, i - r * half, p, q);
+    const int before = r ? r - 1 : m - 2;
+    auto mate = [&](int x, int& pair) {   // partner and pair of player x in the round before
+      int e = x == m - 1 ? 0 : x - before;
+      if (e < 0) e += m - 1;
+      pair = e < half ? e : m - 1 - e;
+      int y, z;
+      pair_of(m, before, pair, y, z);
+      return x == y ? z : y;
+    };
+    int pp, qp;
+    const int pm = mate(p, pp), qm = mate(q, qp);
+    sh.low_bits[i] = uint32_t(p | q << 6 | pm << 12 | qm << 18);
+    sh.high_bits[i] = uint32_t(pp | qp << 6);
   }
   __syncthreads();
-  const int m = (k + 1) & ~1, half = m / 2;
   const int inv = 65536 / max(half, 1) + 1;   // x / half = (x inv) >> 16 for x < half^2 <= 1024
   int buf = 0;
-  bool pending = false;   // rotations of buffer buf ^ 1 not yet applied to V
-  for (int sweep = 0; k > 1 && sweep < 40; ++sweep) {
-    bool done = false;
-    for (int r = 0; r < m - 1; ++r) {
-      if (warp == 0) {
-        int p, q;
-        pair_of(m, r, min(lane, half - 1), p, q);
-        const bool bye = q >= k;
-        double c, s;
-        rotation(0xffffffffu, A[p * k + p], bye ? 0.0 : A[q * k + q], bye ? 0.0 : A[p * k + q], c, s);
-        if (lane < half) {
-          sh.p[buf][lane] = p;
-          sh.q[buf][lane] = q;
-          sh.c[buf][lane] = c;
-          sh.s[buf][lane] = s;
-        }
-      } else {
-        if (pending) rotate_v(V, k, half, sh, buf ^ 1, tid - 32, kThr - 32);
-        if (r == 0) {   // off-diagonal Frobenius norm against the full norm
-          double off = 0.0, tot = 0.0;
-          for (int i = tid - 32; i < k * k; i += kThr - 32) {
-            const double a = A[i];
-            tot = fma(a, a, tot);
-            if (i / k != i % k) off = fma(a, a, off);
+  if (k > 1 && !converged()) {
+    if (warp == 0) round_rotations(A, k, half, 0, false, sh, 0);
+    __syncthreads();
+    for (int sweep = 0; sweep < 40; ++sweep) {
+      for (int r = 0; r < m - 1; ++r) {
+        const bool last = r == m - 2;
+        if (warp == 0) {
+          round_rotations(A, k, half, last ? 0 : r + 1, true, sh, buf ^ 1);
+        } else {
+          // B <- P^T A P: rows of pair a, columns of pair b; lane bit 1 = row, bit 0 = column of
+          // the block (whole groups of four lanes take part)
+          const int nel = 4 * half * half;
+          for (int e0 = (tid & ~31) - 32; e0 < nel; e0 += kThr - 32) {
+            const int e = e0 + lane;
+            const int blk = min(e, nel - 1) >> 2, a = (blk * inv) >> 16, b = blk - a * half;
+            const bool lo = tid & 2, right = tid & 1;
+            const int pa = sh.p[buf][a], qa = sh.q[buf][a], pb = sh.p[buf][b], qb = sh.q[buf][b];
+            const bool ra = qa < k, rb = qb < k;   // (an odd k has one pair with a bye)
+            const int row = lo ? qa : pa, col = right ? qb : pb;
+            const bool mine = e < nel && row < k && col < k;
+            double x = mine ? A[row * k + col] : 0.0;
+            const double sa = sh.s[buf][a], ca = sh.c[buf][a];
+            const double up = __shfl_xor_sync(0xffffffffu, x, 2);
+            if (ra && !is_zero(sa)) x = rotated(lo ? up : x, lo ? x : up, ca, sa, lo);
+            const double sb = sh.s[buf][b], cb = sh.c[buf][b];
+            const double side = __shfl_xor_sync(0xffffffffu, x, 1);
+            if (rb && !is_zero(sb)) x = rotated(right ? side : x, right ? x : side, cb, sb, right);
+            if (mine) {
+              B[row * k + col] = x;
+              if (last) norms(x, row == col);
+            }
           }
-          for (int o = 16; o > 0; o >>= 1) {
-            off += __shfl_xor_sync(0xffffffffu, off, o);
-            tot += __shfl_xor_sync(0xffffffffu, tot, o);
-          }
-          if (lane == 0) {
-            sh.off[warp] = off;
-            sh.tot[warp] = tot;
+          for (int e = tid - 32; e < half * k; e += kThr - 32) {   // V <- V P
+            const int a = e / k, row = e - a * k;
+            const int p = sh.p[buf][a], q = sh.q[buf][a];
+            const double c = sh.c[buf][a], s = sh.s[buf][a];
+            if (q >= k || is_zero(s)) continue;
+            const double vp = V[row * k + p], vq = V[row * k + q];
+            V[row * k + p] = fma(c, vp, -(s * vq));
+            V[row * k + q] = fma(s, vp, c * vq);
           }
         }
+        if (last) norms_out();
+        __syncthreads();
+        double* t = A;
+        A = B;
+        B = t;
+        buf ^= 1;
       }
-      __syncthreads();
-      pending = false;
-      if (r == 0) {   // the same sums in every thread
-        double off = 0.0, tot = 0.0;
-        for (int x = 1; x < kWarps; ++x) {
-          off += sh.off[x];
-          tot += sh.tot[x];
-        }
-        done = off <= 1e-30 * tot || tot == 0.0;
-        if (done) break;
-      }
-      // A <- P^T A P: rows of pair a, columns of pair b; lane bit 1 = row, bit 0 = column of the
-      // block (whole groups of four lanes take part)
-      const int nel = 4 * half * half;
-      for (int e0 = tid & ~31; e0 < nel; e0 += kThr) {   // (whole warps)
-        const int e = e0 + lane;
-        const int blk = min(e, nel - 1) >> 2, a = (blk * inv) >> 16, b = blk - a * half;
-        const bool lo = tid & 2, right = tid & 1;
-        const int pa = sh.p[buf][a], qa = sh.q[buf][a], pb = sh.p[buf][b], qb = sh.q[buf][b];
-        const bool ra = qa < k, rb = qb < k;   // (an odd k has one pair with a bye)
-        const int row = lo ? qa : pa, col = right ? qb : pb;
-        const bool mine = e < nel && row < k && col < k;
-        double x = mine ? A[row * k + col] : 0.0;
-        // row p: c x_p - s x_q, row q: s x_p + c x_q (first product fused, second rounded)
-        const double sa = sh.s[buf][a], ca = sh.c[buf][a];
-        const double up = __shfl_xor_sync(0xffffffffu, x, 2);
-        if (ra && !is_zero(sa))
-          x = fma(lo ? sa : ca, lo ? up : x, flip_if((lo ? ca : sa) * (lo ? x : up), !lo));
-        const double sb = sh.s[buf][b], cb = sh.c[buf][b];
-        const double side = __shfl_xor_sync(0xffffffffu, x, 1);
-        if (rb && !is_zero(sb))
-          x = fma(right ? sb : cb, right ? side : x,
-                  flip_if((right ? cb : sb) * (right ? x : side), !right));
-        if (mine) A[row * k + col] = x;
-      }
-      pending = true;
-      buf ^= 1;
+      if (converged()) break;   // (the rotations formed ahead are dropped)
       __syncthreads();
     }
-    if (done) break;
   }
-  if (pending) rotate_v(V, k, half, sh, buf ^ 1, tid, kThr);
   if (tid < k) sh.w[tid] = A[tid * k + tid];
   if (tid < 2) sh.low[tid] = min(tid, k - 1);   // (stays only if the weights are NaN)
   __syncthreads();
@@ -526,11 +621,11 @@ static size_t ritz_smem(int k) {
   DMRG_REQUIRE(k >= 1 && k <= kMaxK, DMRG_EINVAL, "internal: Ritz problem too large");
   static std::once_flag once;
   std::call_once(once, [] {
-    const int most = int(sizeof(double) * 2 * kMaxK * kMaxK);
+    const int most = int(sizeof(double) * 3 * kMaxK * kMaxK);
     DMRG_CUDA(cudaFuncSetAttribute(k_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     DMRG_CUDA(cudaFuncSetAttribute(k_dav_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
   });
-  return sizeof(double) * 2 * size_t(k) * k;
+  return sizeof(double) * 3 * size_t(k) * k;
 }
 
 void multidot(const double* const* d_vecs, int k, const double* w, int64_t n, double* d_out,
