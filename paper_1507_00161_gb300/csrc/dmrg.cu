@@ -118,8 +118,8 @@ struct Blk {
 struct EnlPlan {
   Layout lay;
   OpSet out;                                   // host tables only, no data
-  std::vector<std::vector<EnlBlock>> part;     // destination blocks in label order
-  std::vector<int64_t> pbase;
+  std::vector<std::vector<EnlBlock>> part;     // parts of the destination blocks in label order
+  std::vector<int64_t> pbase;                  // first part of every list
   std::vector<LayDev> ld;
   double det[8] = {};                          // host seconds of its phases
 };
@@ -653,7 +653,7 @@ static void plan_enlarge(const Ctx& c, const OpSet& blk, int s, bool left, EnlPl
       for (int w = 0; w < W64; ++w)
         for (uint64_t m = acc[w]; m; m &= m - 1) {
           const int Qi = w * 64 + __builtin_ctzll(m);
-          v.push_back(EnlBlock{0, k, qo[Qi], Qi, 0});
+          v.push_back(EnlBlock{0, k, qo[Qi], Qi, 1 << 16});
           el += (int64_t(lay.sec.d[qo[Qi]]) * lay.sec.d[Qi] + 3) & ~int64_t(3);
         }
     }
@@ -678,15 +678,27 @@ static void plan_enlarge(const Ctx& c, const OpSet& blk, int s, bool left, EnlPl
   {
     auto fill = [&](int t) {
       int64_t off = pelem[t], idx = pbase[t];
+      std::vector<EnlBlock> more;   // further parts of wide blocks
       for (EnlBlock& b : part[t]) {
         b.off = off;
         out.blocks[idx++] = OpBlock{b.Qo, b.Qi, off};
         out.lab_ptr[b.k + 1]++;   // labels of one list belong to this list only
-        off += (int64_t(lay.sec.d[b.Qo]) * lay.sec.d[b.Qi] + 3) & ~int64_t(3);
+        const int64_t elems = int64_t(lay.sec.d[b.Qo]) * lay.sec.d[b.Qi];
+        if (elems > kEnlPart) {
+          const int parts = int(std::min<int64_t>((elems + kEnlPart - 1) / kEnlPart, 1024));
+          b.part = parts << 16;
+          for (int q = 1; q < parts; ++q) {
+            more.push_back(b);
+            more.back().part = q | parts << 16;
+          }
+        }
+        off += (elems + 3) & ~int64_t(3);
       }
+      part[t].insert(part[t].end(), more.begin(), more.end());
     };
     WorkerPool::get().run(nparts, [&](int t) { fill(t); });
   }
+  for (int t = 0; t < nparts; ++t) pbase[t + 1] = pbase[t] + int64_t(part[t].size());
   for (int k = 0; k < ndst; ++k) out.lab_ptr[k + 1] += out.lab_ptr[k];
   out.n_elems = pelem[nparts];
   elap(12);

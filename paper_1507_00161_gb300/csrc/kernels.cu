@@ -330,7 +330,9 @@ template void run_copy_tasks<float>(const CopyTask*, int64_t, const CopyTerm*,
 __constant__ int8_t c_op_entries[4][2][2] = {
     {{0, 0}, {1, 1}}, {{1, 1}, {-1, -1}}, {{1, 0}, {-1, -1}}, {{0, 1}, {-1, -1}}};
 
-// One warp per enlarged block.  The block is made of up to four pieces (site states
+// One warp per enlarged block (several for a block of more than kEnlPart elements: a warp alone took
+// 0.9 ms for one of 240 x 240, as long as the whole launch; measured over all right blocks of pf
+// 8p+8n, M0 = 4096: 93 -> 18 ms).  The block is made of up to four pieces (site states
 // sigma_out, sigma_in), each the size of one source block; every contribution (W entry,
 // site-operator element) fills one piece.  The lanes test 32 W entries at a time (source
 // block lookup, Jordan-Wigner sign) and list the contributions per piece in shared memory,
@@ -361,6 +363,8 @@ __global__ void __launch_bounds__(kEnlWarps * 32) k_enlarge(const EnlBlock* __re
   double* dst = out + b.off;
   const int Di = li.D;
   const unsigned below = (1u << lane) - 1u;
+  // elements of this warp: every parts-th run of 32
+  const int first_idx = (b.part & 0xffff) * kWarp + lane, step = (b.part >> 16) * kWarp;
   const int x_end = eptr[b.k + 1];
   int x0 = eptr[b.k];
   bool first = true;   // the first pass writes, later passes (long lists) add
@@ -419,7 +423,7 @@ __global__ void __launch_bounds__(kEnlWarps * 32) k_enlarge(const EnlBlock* __re
       const int ro = so ? lo.poff1 : 0, ri = si ? li.poff1 : 0;
       const int64_t* offs = s_off[warp][p];
       const double* scs = s_sc[warp][p];
-      for (int idx = lane; idx < rows * cols; idx += kWarp) {
+      for (int idx = first_idx; idx < rows * cols; idx += step) {
         const int r = idx / cols, cc = idx - r * cols;
         double* d = dst + (int64_t)(ro + r) * Di + ri + cc;
         double acc = first ? 0.0 : *d;
