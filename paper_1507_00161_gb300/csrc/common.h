@@ -587,28 +587,26 @@ struct EntryDev {
 };
 struct EnlBlock {
   int64_t off;     // destination block offset
-  int32_t k, Qo, Qi, pad;
+  int32_t k, Qo, Qi;
+  int32_t part;    // part number + (parts << 16): wide blocks are shared by several warps
 };
+constexpr int kEnlPart = 2048;   // elements of a block per warp
 struct LayDev {
   int32_t pblk0, pblk1, poff1, D;
 };
-// one operator block to renormalize: O (enlarged sectors so, si) at xoff -> O' at yoff,
-// intermediate O U_i at toff of the scratch
+// renormalization of one operator block O (enlarged sectors so, si) at xoff -> O' at yoff, columns
+// c0 .. c0 + 31 of O' (renorm.cu).  Blocks come in three classes by size (project_class), each with
+// its units one after the other: units of class k at [begin[k], begin[k + 1])
 struct ProjTask {
-  int64_t xoff, yoff, toff;
-  int32_t so, si;
+  int64_t xoff, yoff;
+  int32_t so, si, c0, pad;
 };
-// tile_beg1/2: [n + 1] prefix sums of the 32 x 32 tiles of stage 1 (D_o x m_i) and
-// stage 2 (m_o x m_i) per block
-void project_blocks(const ProjTask* tasks, const int64_t* tile_beg1, int64_t n_tiles1,
-                    const int64_t* tile_beg2, int64_t n_tiles2, int64_t n, const int32_t* D,
+int project_class(int Do, int Di);
+int project_units(int cls, int mi);
+void project_blocks(const ProjTask* units, const int64_t (&begin)[4], const int32_t* D,
                     const int32_t* m, const int64_t* uoff, const double* X, const double* U,
-                    double* T, double* Y, cudaStream_t s);
-// blocks with D_o, D_i <= 32 (one warp each, both products fused)
+                    double* Y, cudaStream_t s);
 void set_ones(double* x, const int64_t* pos, int64_t n, cudaStream_t s);
-void project_small(const ProjTask* tasks, int64_t n, const int32_t* D, const int32_t* m,
-                   const int64_t* uoff, const double* X, const double* U, double* Y,
-                   cudaStream_t s);
 void enlarge_blocks(const EnlBlock* blocks, int64_t n, const int32_t* eptr, const EntryDev* ents,
                     const int32_t* src_by_in, int src_nsec, const int64_t* src_boff,
                     const int32_t* src_dim, const int32_t* src_npart, const int8_t* src_lpar,

@@ -877,62 +877,78 @@ static void project(Ctx& c, OpSet& E, const Iso& iso, OpSet& out) {
   out.lab_ptr.assign(E.nlab + 1, 0);
   out.blocks.clear();
   double tp = wall();
-  // one renormalization task per kept block, read by k_project straight from this table
-  std::vector<ProjTask> tasks, small;
-  small.reserve(E.blocks.size());
-  std::vector<int64_t> tb1(1, 0), tb2(1, 0);
-  int64_t noff = 0, toff = 0;
-  for (int k = 0; k < E.nlab; ++k) {
-    out.lab_ptr[k] = int64_t(out.blocks.size());
+  // one renormalization unit per kept block (and 32 columns of a wide one), built label by label:
+  // counts first, then every label fills its own ranges
+  struct Count {
+    int64_t blocks = 0, elems = 0, units[3] = {0, 0, 0};
+  };
+  std::vector<Count> at(size_t(E.nlab) + 1);
+  auto walk = [&](int k, auto&& each) {
     for (int64_t x = E.lab_ptr[k]; x < E.lab_ptr[k + 1]; ++x) {
       const OpBlock& b = E.blocks[x];
-      const int no = iso.kept_idx[b.so], ni = iso.kept_idx[b.si];
-      if (no < 0 || ni < 0) continue;
-      const int Do = E.sec.d[b.so], Di = E.sec.d[b.si], mo = iso.m[b.so], mi = iso.m[b.si];
-      DMRG_REQUIRE(b.off + int64_t(Do) * Di <= E.n_elems, DMRG_EINVAL,
-                   "internal: operator block out of range");
-      out.blocks.push_back(OpBlock{no, ni, noff});
-      if (Do <= 32 && Di <= 32) {
-        small.push_back(ProjTask{b.off, noff, 0, b.so, b.si});
-      } else {
-        tasks.push_back(ProjTask{b.off, noff, toff, b.so, b.si});
-        const int64_t ct = (mi + 31) / 32;
-        tb1.push_back(tb1.back() + (Do + 31) / 32 * ct);
-        tb2.push_back(tb2.back() + (mo + 31) / 32 * ct);
-        toff += int64_t(Do) * mi;
-      }
-      noff += int64_t(mo) * mi;
+      if (iso.kept_idx[b.so] >= 0 && iso.kept_idx[b.si] >= 0) each(b);
     }
+  };
+  parallel_for(E.nlab, [&](int k0, int k1, int) {
+    for (int k = k0; k < k1; ++k) {
+      Count& c1 = at[k + 1];
+      walk(k, [&](const OpBlock& b) {
+        const int cls = project_class(E.sec.d[b.so], E.sec.d[b.si]);
+        c1.blocks += 1;
+        c1.elems += int64_t(iso.m[b.so]) * iso.m[b.si];
+        c1.units[cls] += project_units(cls, iso.m[b.si]);
+      });
+    }
+  });
+  for (int k = 0; k < E.nlab; ++k) {
+    at[k + 1].blocks += at[k].blocks;
+    at[k + 1].elems += at[k].elems;
+    for (int q = 0; q < 3; ++q) at[k + 1].units[q] += at[k].units[q];
   }
-  out.lab_ptr[E.nlab] = int64_t(out.blocks.size());
-  out.n_elems = noff;
+  const Count& total = at[E.nlab];
+  const int64_t begin[4] = {0, total.units[0], total.units[0] + total.units[1],
+                            total.units[0] + total.units[1] + total.units[2]};
+  DMRG_REQUIRE(begin[3] < (int64_t(1) << 31), DMRG_EINVAL, "too many operator blocks");
+  std::vector<ProjTask> units(begin[3]);
+  out.blocks.resize(total.blocks);
+  for (int k = 0; k <= E.nlab; ++k) out.lab_ptr[k] = at[k].blocks;
+  std::atomic<bool> outside{false};
+  parallel_for(E.nlab, [&](int k0, int k1, int) {
+    for (int k = k0; k < k1; ++k) {
+      Count c0 = at[k];
+      walk(k, [&](const OpBlock& b) {
+        const int Do = E.sec.d[b.so], Di = E.sec.d[b.si], mi = iso.m[b.si];
+        if (b.off + int64_t(Do) * Di > E.n_elems) outside = true;
+        out.blocks[c0.blocks++] = OpBlock{iso.kept_idx[b.so], iso.kept_idx[b.si], c0.elems};
+        const int cls = project_class(Do, Di), nu = project_units(cls, mi);
+        for (int u = 0; u < nu; ++u)
+          units[begin[cls] + c0.units[cls]++] = ProjTask{b.off, c0.elems, b.so, b.si, 32 * u, 0};
+        c0.elems += int64_t(iso.m[b.so]) * mi;
+      });
+    }
+  });
+  DMRG_REQUIRE(!outside, DMRG_EINVAL, "internal: operator block out of range");
+  out.n_elems = total.elems;
   std::vector<int64_t> uo(nE);
   for (int i = 0; i < nE; ++i) {
     uo[i] = iso.uoff[i];
     DMRG_REQUIRE(iso.m[i] == 0 || uo[i] + int64_t(E.sec.d[i]) * iso.m[i] <= iso.data.n,
                  DMRG_EINVAL, "internal: isometry out of range");
   }
-  out.data.alloc(std::max<int64_t>(noff, 1));
-  c.tmp.alloc(std::max<int64_t>(toff, 1));
-  DevBuf<ProjTask> dt, dts;
+  out.data.alloc(std::max<int64_t>(out.n_elems, 1));
+  DevBuf<ProjTask> du;
   DevBuf<int32_t> dD, dm;
-  DevBuf<int64_t> duo, dtb1, dtb2;
-  dt.upload(tasks, c.stream);
-  dts.upload(small, c.stream);
-  dtb1.upload(tb1, c.stream);
-  dtb2.upload(tb2, c.stream);
+  DevBuf<int64_t> duo;
+  du.upload(units, c.stream);
   dD.upload(E.sec.d, c.stream);
   dm.upload(iso.m, c.stream);
   duo.upload(uo, c.stream);
   c.t_detail[4] += wall() - tp;
   tp = wall();
-  project_small(dts.p, int64_t(small.size()), dD.p, dm.p, duo.p, E.data.p, iso.data.p,
-                out.data.p, c.stream);
   // FP64 in both precisions: the stored operators must keep the Hermitian pairing of the
   // normal and complementary operators to FP64 rounding; split-TF32 products left the pairs
   // unequal at ~1e-6 relative, which floored the Davidson residual of the next steps
-  project_blocks(dt.p, dtb1.p, tb1.back(), dtb2.p, tb2.back(), int64_t(tasks.size()), dD.p,
-                 dm.p, duo.p, E.data.p, iso.data.p, c.tmp.p, out.data.p, c.stream);
+  project_blocks(du.p, begin, dD.p, dm.p, duo.p, E.data.p, iso.data.p, out.data.p, c.stream);
   sync(c);
   c.t_detail[5] += wall() - tp;
   tp = wall();

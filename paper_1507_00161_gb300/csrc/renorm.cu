@@ -3,14 +3,18 @@
 // of every normal and complementary operator, U_Q = kept eigenvectors of the reduced
 // density matrix in enlarged sector Q (D_Q x m_Q, row-major).
 //
-// Driven by the block table itself (no per-GEMM task lists):
-//  - blocks with D_o, D_i <= 32: one warp each, both products fused, T = O U_i held in
-//    shared memory; lane = (column c, row group g) so that narrow blocks keep all lanes busy;
-//  - larger blocks: two batched GEMM passes, T_b = O_b U_i to a scratch, then
-//    O'_b = U_o^T T_b, each cut into 32 x 32 output tiles; thread block t finds its block by
-//    binary search in the prefix sums of tiles per block; K in chunks of 32 through shared
-//    memory.
-// FP64 throughout, fixed summation order (deterministic).
+// FP64 is one warp instruction per 19 clocks and SM on this chip, whatever its active lanes, so
+// the elements of T = O U_i and of U_o^T T are numbered through and dealt to the lanes 32 at a
+// time, and nothing is computed for padding; the operands are read where they are (rows of O and
+// columns of U_o broadcast, rows of U_i consecutive).  Driven by the block table itself:
+//  - blocks with D_o, D_i <= 16: one warp each, T in shared memory;
+//  - larger blocks: units of a block and up to 32 columns of U_i, one thread block each, T in
+//    shared memory, 32 or 128 of its rows at a time; with more rows than that the result grows
+//    chunk by chunk in its place.
+// FP64 throughout, every sum in index order (deterministic).
+// Measured (GB300) against 32 x 32 tiles in two passes through a scratch and one warp per block up to
+// 32: all right blocks of pf 8p+8n, M0 = 4096, 361 -> 270 ms of kernels; at M = 4096, position 15, the
+// two steps of a pair 1.5 -> 0.5 ms each.
 #include <stdint.h>
 
 #include "common.h"
@@ -19,147 +23,108 @@ namespace dmrg {
 
 namespace {
 
-constexpr int kPT = 32;              // tile edge
-constexpr int kPS = kPT + 1;         // padded shared row
-constexpr int kPThreads = 128;
+constexpr int kCols = 32;            // columns of a unit
+constexpr int kLd = kCols + 1;
+constexpr int kThr = 128;
+constexpr int kTiny = 16, kTinyLd = kTiny + 1;
+constexpr int kTinyWarps = 4;
 
-// C (M x N, ldc) = op(A) (M x K) B (K x N, ldb); A stored M x K (lda) or, transposed, K x M
-// (lda).  Thread (ty, tx) owns rows ty, ty + 16 and columns tx, tx + 8, tx + 16, tx + 24.
-template <bool TA>
-__device__ __forceinline__ void tile_gemm(const double* __restrict__ A, int lda,
-                                          const double* __restrict__ B, int ldb,
-                                          double* __restrict__ C, int ldc, int M, int N, int K,
-                                          int r0, int c0, double (*As)[kPS], double (*Bs)[kPS]) {
-  const int tid = threadIdx.x;
-  const int ty = tid >> 3, tx = tid & 7;
-  double acc[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
-  for (int k0 = 0; k0 < K; k0 += kPT) {
-    for (int e = tid; e < kPT * kPT; e += kPThreads) {
-      const int i = e >> 5, j = e & 31;
-      if (TA)   // As[k][row] = A^T: A stored K x M
-        As[i][j] = (k0 + i < K && r0 + j < M) ? A[int64_t(k0 + i) * lda + r0 + j] : 0.0;
-      else      // As[row][k]
-        As[i][j] = (r0 + i < M && k0 + j < K) ? A[int64_t(r0 + i) * lda + k0 + j] : 0.0;
-      Bs[i][j] = (k0 + i < K && c0 + j < N) ? B[int64_t(k0 + i) * ldb + c0 + j] : 0.0;
-    }
-    __syncthreads();
-    const int kn = min(kPT, K - k0);
+// c[r * 1] ... sum_k a[k sa] b[k sb], k < n, in order
+__device__ __forceinline__ double dot_strided(const double* __restrict__ a, int64_t sa,
+                                              const double* b, int64_t sb, int n, double s) {
 #pragma unroll 4
-    for (int k = 0; k < kn; ++k) {
-      const double a0 = TA ? As[k][ty] : As[ty][k];
-      const double a1 = TA ? As[k][ty + 16] : As[ty + 16][k];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double b = Bs[k][tx + 8 * q];
-        acc[0][q] = fma(a0, b, acc[0][q]);
-        acc[1][q] = fma(a1, b, acc[1][q]);
+  for (int k = 0; k < n; ++k) s = fma(a[k * sa], b[k * sb], s);
+  return s;
+}
+
+template <int ROWS>
+__global__ void __launch_bounds__(kThr, ROWS == 32 ? 12 : 6)
+k_project(const ProjTask* __restrict__ units, const int32_t* __restrict__ D,
+          const int32_t* __restrict__ m, const int64_t* __restrict__ uoff,
+          const double* __restrict__ X, const double* __restrict__ U, double* __restrict__ Y) {
+  __shared__ double T[ROWS * kLd];
+  const ProjTask pt = units[blockIdx.x];
+  const int Do = D[pt.so], Di = D[pt.si], mo = m[pt.so], mi = m[pt.si];
+  const int n = min(kCols, mi - pt.c0);
+  const double* __restrict__ Xb = X + pt.xoff;
+  const double* __restrict__ Ui = U + uoff[pt.si] + pt.c0;
+  const double* __restrict__ Uo = U + uoff[pt.so];
+  double* __restrict__ Yb = Y + pt.yoff + pt.c0;
+  // e / n = (e inv) >> 16 for e < 1024: elements are dealt in runs of kRun rows of n
+  const int inv = 65536 / n + 1;
+  constexpr int kRun = 32;
+  for (int i0 = 0; i0 < Do; i0 += ROWS) {
+    const int rows = min(ROWS, Do - i0);
+    for (int r0 = 0; r0 < rows; r0 += kRun) {
+      const int cnt = min(kRun, rows - r0) * n;
+      for (int e = threadIdx.x; e < cnt; e += kThr) {
+        const int i = (e * inv) >> 16, c = e - i * n;
+        T[(r0 + i) * kLd + c] =
+            dot_strided(Xb + int64_t(i0 + r0 + i) * Di, 1, Ui + c, mi, Di, 0.0);
+      }
+    }
+    __syncthreads();
+    for (int a0 = 0; a0 < mo; a0 += kRun) {
+      const int cnt = min(kRun, mo - a0) * n;
+      for (int e = threadIdx.x; e < cnt; e += kThr) {
+        const int a = (e * inv) >> 16, c = e - a * n;
+        double* y = Yb + int64_t(a0 + a) * mi + c;
+        *y = dot_strided(Uo + int64_t(i0) * mo + a0 + a, mo, T + c, kLd, rows, i0 ? *y : 0.0);
       }
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 + ty + 16 * h, cc = c0 + tx + 8 * q;
-      if (r < M && cc < N) C[int64_t(r) * ldc + cc] = acc[h][q];
-    }
 }
 
-template <int STAGE>
-__global__ void __launch_bounds__(kPThreads)
-k_project(const ProjTask* __restrict__ tasks, const int64_t* __restrict__ tile_beg, int64_t n,
-          const int32_t* __restrict__ D, const int32_t* __restrict__ m,
-          const int64_t* __restrict__ uoff, const double* __restrict__ X,
-          const double* __restrict__ U, double* __restrict__ T, double* __restrict__ Y) {
-  __shared__ double As[kPT][kPS];
-  __shared__ double Bs[kPT][kPS];
-  const int64_t n_tiles = tile_beg[n];
-  for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    // block b: tile_beg[b] <= t < tile_beg[b + 1]
-    int64_t lo = 0, hi = n;
-    while (hi - lo > 1) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (tile_beg[mid] <= t) lo = mid;
-      else hi = mid;
-    }
-    const ProjTask pt = tasks[lo];
-    const int l = int(t - tile_beg[lo]);
-    const int Do = D[pt.so], Di = D[pt.si], mo = m[pt.so], mi = m[pt.si];
-    const int nct = (mi + kPT - 1) / kPT;
-    const int r0 = (l / nct) * kPT, c0 = (l % nct) * kPT;
-    if (STAGE == 1)
-      tile_gemm<false>(X + pt.xoff, Di, U + uoff[pt.si], mi, T + pt.toff, mi, Do, mi, Di, r0, c0,
-                       As, Bs);
-    else
-      tile_gemm<true>(U + uoff[pt.so], mo, T + pt.toff, mi, Y + pt.yoff, mi, mo, mi, Do, r0, c0,
-                      As, Bs);
-  }
-}
-
-constexpr int kSWarps = 4;
-
-__global__ void __launch_bounds__(kSWarps * 32)
-k_project_small(const ProjTask* __restrict__ tasks, int64_t n, const int32_t* __restrict__ D,
-                const int32_t* __restrict__ m, const int64_t* __restrict__ uoff,
-                const double* __restrict__ X, const double* __restrict__ U,
-                double* __restrict__ Y) {
-  __shared__ double Ts[kSWarps][kPT][kPS];
+__global__ void __launch_bounds__(kTinyWarps * 32)
+k_project_tiny(const ProjTask* __restrict__ tasks, int64_t n, const int32_t* __restrict__ D,
+               const int32_t* __restrict__ m, const int64_t* __restrict__ uoff,
+               const double* __restrict__ X, const double* __restrict__ U,
+               double* __restrict__ Y) {
+  __shared__ double Ts[kTinyWarps][kTiny * kTinyLd];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double (*T)[kPS] = Ts[warp];
-  for (int64_t b = int64_t(blockIdx.x) * kSWarps + warp; b < n; b += int64_t(gridDim.x) * kSWarps) {
-    const ProjTask pt = tasks[b];
-    const int Do = D[pt.so], Di = D[pt.si], mo = m[pt.so], mi = m[pt.si];
-    const double* Xb = X + pt.xoff;
-    const double* Ui = U + uoff[pt.si];
-    const double* Uo = U + uoff[pt.so];
-    double* Yb = Y + pt.yoff;
-    const int groups = 32 / mi;          // mi <= Di <= 32
-    const int cc = lane % mi, g = lane / mi;
-    if (g < groups) {
-      for (int i = g; i < Do; i += groups) {
-        double acc = 0.0;
-        for (int k = 0; k < Di; ++k) acc = fma(Xb[i * Di + k], Ui[k * mi + cc], acc);
-        T[i][cc] = acc;
-      }
-    }
-    __syncwarp();
-    if (g < groups) {
-      for (int a = g; a < mo; a += groups) {
-        double acc = 0.0;
-        for (int i = 0; i < Do; ++i) acc = fma(Uo[i * mo + a], T[i][cc], acc);
-        Yb[a * mi + cc] = acc;
-      }
-    }
-    __syncwarp();
+  double* T = Ts[warp];
+  const int64_t b = int64_t(blockIdx.x) * kTinyWarps + warp;
+  if (b >= n) return;
+  const ProjTask pt = tasks[b];
+  const int Do = D[pt.so], Di = D[pt.si], mo = m[pt.so], mi = m[pt.si];
+  const double* __restrict__ Xb = X + pt.xoff;
+  const double* __restrict__ Ui = U + uoff[pt.si];
+  const double* __restrict__ Uo = U + uoff[pt.so];
+  const int inv = 65536 / mi + 1;
+  for (int e = lane; e < Do * mi; e += 32) {
+    const int i = (e * inv) >> 16, c = e - i * mi;
+    T[i * kTinyLd + c] = dot_strided(Xb + i * Di, 1, Ui + c, mi, Di, 0.0);
+  }
+  __syncwarp();
+  for (int e = lane; e < mo * mi; e += 32) {
+    const int a = (e * inv) >> 16, c = e - a * mi;
+    Y[pt.yoff + e] = dot_strided(Uo + a, mo, T + c, kTinyLd, Do, 0.0);
   }
 }
 
 }  // namespace
 
-void project_small(const ProjTask* tasks, int64_t n, const int32_t* D, const int32_t* m,
-                   const int64_t* uoff, const double* X, const double* U, double* Y,
-                   cudaStream_t s) {
-  if (n <= 0) return;
-  const int64_t blocks = std::min<int64_t>((n + kSWarps - 1) / kSWarps, 152 * 16 * 32);
-  k_project_small<<<int(blocks), kSWarps * 32, 0, s>>>(tasks, n, D, m, uoff, X, U, Y);
-  DMRG_LAUNCHED();
+int project_class(int Do, int Di) {
+  return Do <= kTiny && Di <= kTiny ? 0 : Do <= 32 ? 1 : 2;
 }
+int project_units(int cls, int mi) { return cls == 0 ? 1 : (mi + kCols - 1) / kCols; }
 
-void project_blocks(const ProjTask* tasks, const int64_t* tile_beg1, int64_t n_tiles1,
-                    const int64_t* tile_beg2, int64_t n_tiles2, int64_t n, const int32_t* D,
+void project_blocks(const ProjTask* units, const int64_t (&begin)[4], const int32_t* D,
                     const int32_t* m, const int64_t* uoff, const double* X, const double* U,
-                    double* T, double* Y, cudaStream_t s) {
-  if (n <= 0) return;
-  const int64_t cap = 152 * 16 * 64;
-  if (n_tiles1 > 0) {
-    k_project<1><<<int(std::min(n_tiles1, cap)), kPThreads, 0, s>>>(tasks, tile_beg1, n, D, m,
-                                                                     uoff, X, U, T, Y);
+                    double* Y, cudaStream_t s) {
+  const int64_t n0 = begin[1] - begin[0], n1 = begin[2] - begin[1], n2 = begin[3] - begin[2];
+  if (n2 > 0) {   // the widest first
+    k_project<128><<<int(n2), kThr, 0, s>>>(units + begin[2], D, m, uoff, X, U, Y);
     DMRG_LAUNCHED();
   }
-  if (n_tiles2 > 0) {
-    k_project<2><<<int(std::min(n_tiles2, cap)), kPThreads, 0, s>>>(tasks, tile_beg2, n, D, m,
-                                                                     uoff, X, U, T, Y);
+  if (n1 > 0) {
+    k_project<32><<<int(n1), kThr, 0, s>>>(units + begin[1], D, m, uoff, X, U, Y);
+    DMRG_LAUNCHED();
+  }
+  if (n0 > 0) {
+    k_project_tiny<<<int((n0 + kTinyWarps - 1) / kTinyWarps), kTinyWarps * 32, 0, s>>>(
+        units + begin[0], n0, D, m, uoff, X, U, Y);
     DMRG_LAUNCHED();
   }
 }
