@@ -155,13 +155,16 @@ k_heff_reduce_slots(const HeffRed* __restrict__ red, int64_t n_plain, const Heff
   const T* __restrict__ P = ptrs.P[r.inst] + (plain ? r.poff : r.qoff);
   T* __restrict__ Y = ptrs.Y[r.inst];
   const int mn = r.m * r.n;
-  for (int e = threadIdx.x; e < mn; e += blockDim.x) {
+  // the outputs of a tile are spread over blockIdx.y: a tile has few of them and many addends
+  // (one block per tile took 28 us for 900 tiles, four take 10)
+  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < mn; e += gridDim.y * blockDim.x) {
     T s = T(0);
+    if (plain) {
 #pragma unroll 4
-    for (int g = 0; g < r.groups; ++g) {
-      if (plain) {
-        s += P[int64_t(g) * mn + e];
-      } else {
+      for (int g = 0; g < r.groups; ++g) s += P[int64_t(g) * mn + e];
+    } else {
+#pragma unroll 4
+      for (int g = 0; g < r.groups; ++g) {
         const T* q = P + int64_t(g) * kSlots * mn + e;
         T u = q[0];
 #pragma unroll
@@ -216,7 +219,7 @@ template <class T>
 void heff_reduce_slots(const HeffRed* d_red, int64_t n_plain, int64_t n_red, const HeffPtrs<T>& ptrs,
                        cudaStream_t s) {
   if (n_red <= 0) return;
-  k_heff_reduce_slots<T><<<int(n_red), 128, 0, s>>>(d_red, n_plain, ptrs);
+  k_heff_reduce_slots<T><<<dim3(unsigned(n_red), 4), 128, 0, s>>>(d_red, n_plain, ptrs);
   DMRG_LAUNCHED();
 }
 template void heff_reduce_slots<float>(const HeffRed*, int64_t, int64_t, const HeffPtrs<float>&,
