@@ -671,10 +671,9 @@ void batched_eigh2(const int64_t* d_off, const int64_t* d_woff, const int32_t* d
 // bitonic sort (descending) of w padded to np2 with -inf, in shared memory when it fits
 constexpr int64_t kKthSmem = 16384;
 
-// out[0] = the k-th largest weight.  Fixed count (target <= 0): k = kmax.  Dynamic block
-// state selection (target > 0): k = the smallest count in [kmin, kmax] whose discarded
-// weight 1 - (w_1 + ... + w_k) (sorted descending, summed in that order in FP64) is at
-// most target, else kmax.  out[1] = k.
+// out[0] = the k-th largest weight, out[1] = k, for dynamic block state selection: k = the
+// smallest count in [kmin, kmax] whose discarded weight 1 - (w_1 + ... + w_k) (sorted descending,
+// summed in that order in FP64) is at most target, else kmax.
 __global__ void k_kth_largest(const double* __restrict__ w, int64_t n, int64_t kmax, int64_t kmin,
                               double target, double* gbuf, int64_t np2, double* out) {
   extern __shared__ double kth_sm[];
@@ -713,9 +712,69 @@ __global__ void k_kth_largest(const double* __restrict__ w, int64_t n, int64_t k
     out[1] = double(k);
   }
 }
+// The k-th largest of n values alone (a fixed count): their order is the order of their bits as
+// unsigned integers once negative ones are inverted, and the value is found 8 bits at a time from a
+// histogram of the values that share the bits found so far.  Exact.  A sort in one block took
+// 385 us for 8000 weights and 1957 us for 30000, this 18 and 47 us; for 128 it is 10 against 14 us.
+__device__ __forceinline__ unsigned long long order_key(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return b >> 63 ? ~b : b | 0x8000000000000000ull;
+}
+constexpr int kHists = 8;   // histograms side by side: fewer collisions
+__global__ void __launch_bounds__(1024) k_select(const double* __restrict__ w, int64_t n, int64_t k,
+                                                 double* __restrict__ out) {
+  __shared__ int hist[kHists][256], s_warp[8], s_digit, s_rest;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned long long prefix = 0;
+  int rest = int(k);
+  for (int shift = 56; shift >= 0; shift -= 8) {
+    for (int i = tid; i < kHists * 256; i += 1024) hist[i >> 8][i & 255] = 0;
+    __syncthreads();
+    for (int64_t i = tid; i < n; i += 1024) {
+      const unsigned long long key = order_key(w[i]);
+      if (shift == 56 || key >> (shift + 8) == prefix)
+        atomicAdd(&hist[warp % kHists][(key >> shift) & 255], 1);
+    }
+    __syncthreads();
+    // thread d of the first 256: values with the digit 255 - d, and with a larger one
+    int mine = 0, upto = 0;
+    if (tid < 256) {
+      for (int x = 0; x < kHists; ++x) mine += hist[x][255 - tid];
+      upto = mine;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += v;
+      }
+      if (lane == 31) s_warp[warp] = upto;
+    }
+    __syncthreads();
+    if (tid < 256) {
+      for (int x = 0; x < warp; ++x) upto += s_warp[x];
+      if (upto >= rest && upto - mine < rest) {   // exactly one thread: rest <= number of values
+        s_digit = 255 - tid;
+        s_rest = rest - (upto - mine);
+      }
+    }
+    __syncthreads();
+    prefix = prefix << 8 | (unsigned long long)s_digit;
+    rest = s_rest;
+    __syncthreads();
+  }
+  if (tid == 0) {
+    const unsigned long long b = prefix >> 63 ? prefix & 0x7fffffffffffffffull : ~prefix;
+    out[0] = __longlong_as_double((long long)b);
+    out[1] = double(k);
+  }
+}
+
 void kth_largest(const double* w, int64_t n, int64_t kmax, int64_t kmin, double target,
                  double* d_scratch, double* out, cudaStream_t s) {
   DMRG_REQUIRE(kmax >= 1 && kmax <= n && kmin >= 1, DMRG_EINVAL, "internal: bad selection count");
+  if (!(target > 0.0)) {
+    k_select<<<1, 1024, 0, s>>>(w, n, kmax, out);
+    DMRG_LAUNCHED();
+    return;
+  }
   int64_t np2 = 1;
   while (np2 < n) np2 <<= 1;
   static std::once_flag once;
