@@ -25,6 +25,9 @@
 //        c = 1 / sqrt(1 + t^2), s = c t,   a_p <- c a_p - s a_q,  a_q <- s a_p + c a_q
 //      (skipped when |gamma| <= tol sqrt(alpha beta));
 //   3. every CTA rotates its rows.
+// FP64 is one warp instruction per 19 clocks and SM here, so step 1 counts: the lane sums of
+// a warp's pairs run together (31 additions for eight pairs instead of 120), and the rotation's divisions and roots are those of
+// newton.cuh.  Measured (GB300): truncation of pf 8p+8n at M = 4096, position 15, 1.84 -> 1.30 ms.
 // Partial sums are double-buffered, so one cluster barrier per round suffices.  A sweep
 // without a rotation ends the iteration (every CTA takes the same decision); after
 // kMaxSweeps sweeps the job raises the context's non-convergence flag and still writes
@@ -38,6 +41,7 @@
 #include <mutex>
 
 #include "common.h"
+#include "newton.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -92,6 +96,93 @@ __device__ __forceinline__ void round_pair(int m, int r, int k, int& p, int& q) 
   q = max(a, b);
 }
 
+// The sums of V values (a power of two) over the lanes, for each the binary tree over the 32 lanes
+// (l + (l + 16), then 8, 4, 2, 1): after the first level half of the lanes would idle, so two values
+// share an instruction from there on, four from the next.  Lane l ends with the sum of value
+// packed_index(l) mod V.
+template <int V>
+__device__ __forceinline__ double packed_sums(double (&v)[V]) {
+  const int lane = threadIdx.x & 31;
+  int left = V;
+#pragma unroll
+  for (int bit = 16; bit > 0; bit >>= 1) {
+    const bool up = lane & bit;
+    if (left == 1) {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], bit);
+      continue;
+    }
+    left /= 2;
+#pragma unroll
+    for (int i = 0; i < V / 2; ++i)
+      if (i < left)
+        v[i] = (up ? v[2 * i + 1] : v[2 * i]) +
+               __shfl_xor_sync(0xffffffffu, up ? v[2 * i] : v[2 * i + 1], bit);
+  }
+  return v[0];
+}
+__device__ __forceinline__ int packed_index(int lane) { return int(__brev(unsigned(lane)) >> 27); }
+
+// |ga| > tol sqrt(al) sqrt(be): decided by the squares unless they are within 1e-9 of each other
+// or far out in the exponent range (al, be > 0)
+__device__ __forceinline__ bool above(double al, double be, double ga, double tol) {
+  const double l = ga * ga, r = tol * tol * al * be;
+  if (mid_range(l) && mid_range(r) && mid_range(al) && mid_range(be)) {
+    if (l > r * (1.0 + 1e-9)) return true;
+    if (l < r * (1.0 - 1e-9)) return false;
+  }
+  return fabs(ga) > tol * sqrt(al) * sqrt(be);
+}
+
+// zeta = (be - al) / (2 ga), t = sgn(zeta) / (|zeta| + sqrt(1 + zeta^2)), c = 1 / sqrt(1 + t^2),
+// s = c t
+__device__ __forceinline__ void svd_rotation(double al, double be, double ga, double& cs, double& sn) {
+  const double diff = be - al;
+  if (mid_range(ga) && mid_range(diff) && exponent(diff) - exponent(ga) < 180) {
+    const double zeta = quick_div(diff, times_pow2(ga, 1));
+    const double u = quick_rcp(fabs(zeta) + quick_sqrt(fma(zeta, zeta, 1.0)));
+    const double t = flip_if(u, __double2hiint(zeta) < 0);
+    cs = quick_rcp(quick_sqrt(fma(t, t, 1.0)));
+    sn = cs * t;
+    return;
+  }
+  const double zeta = diff / (2.0 * ga);
+  const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+  cs = 1.0 / sqrt(1.0 + t * t);
+  sn = cs * t;
+}
+
+// |a_p|^2, |a_q|^2, a_p . a_q over the nr local rows for the pairs k0, k0 + step, ... (G of them,
+// those below `half`) of round r, into pb[3 k ..]; one warp
+template <int G>
+__device__ __forceinline__ void pair_sums(const double* A, int ld, int nr, int cols, int m, int r,
+                                          int k0, int step, double* pb) {
+  const int lane = threadIdx.x & 31, half = m / 2;
+  double v[4 * G];
+#pragma unroll
+  for (int x = 0; x < G; ++x) {
+    double al = 0.0, be = 0.0, ga = 0.0;
+    const int k = k0 + x * step;
+    if (k < half) {
+      int p, q;
+      round_pair(m, r, k, p, q);
+      if (q < cols)
+        for (int i = lane; i < nr; i += 32) {
+          const double u = A[i * ld + p], w = A[i * ld + q];
+          al = fma(u, u, al);
+          be = fma(w, w, be);
+          ga = fma(u, w, ga);
+        }
+    }
+    v[4 * x] = al;
+    v[4 * x + 1] = be;
+    v[4 * x + 2] = ga;
+    v[4 * x + 3] = 0.0;
+  }
+  const double sum = packed_sums<4 * G>(v);
+  const int at = packed_index(lane), k = k0 + (at >> 2) * step;
+  if (at < 4 * G && (at & 3) < 3 && k < half) pb[3 * k + (at & 3)] = sum;
+}
+
 // NT threads per CTA (256; 64 for single-CTA sectors was measured slower: their rounds are
 // latency-bound, and fewer threads lengthen each round more than the shorter barriers save)
 template <int NT>
@@ -138,29 +229,14 @@ __global__ void __launch_bounds__(NT, 1)
   while (!converged && sweep < kMaxSweeps) {
     if (tid == 0) s_flag = 0;
     for (int r = 0; r < m - 1; ++r) {
-      // 1. partial sums over local rows, one warp per pair
+      // 1. partial sums over local rows, up to eight pairs per warp at a time
       double* pb = part + buf * partN;
-      for (int k = warp; k < m / 2; k += nwarp) {
-        int p, q;
-        round_pair(m, r, k, p, q);
-        double al = 0.0, be = 0.0, ga = 0.0;
-        if (q < S.cols)
-          for (int i = lane; i < nr; i += 32) {
-            const double x = A[i * ld + p], y = A[i * ld + q];
-            al = fma(x, x, al);
-            be = fma(y, y, be);
-            ga = fma(x, y, ga);
-          }
-        for (int o = 16; o > 0; o >>= 1) {
-          al += __shfl_down_sync(0xffffffffu, al, o);
-          be += __shfl_down_sync(0xffffffffu, be, o);
-          ga += __shfl_down_sync(0xffffffffu, ga, o);
-        }
-        if (lane == 0) {
-          pb[3 * k] = al;
-          pb[3 * k + 1] = be;
-          pb[3 * k + 2] = ga;
-        }
+      for (int k0 = warp; k0 < m / 2; k0 += 8 * nwarp) {
+        const int mine = (m / 2 - k0 + nwarp - 1) / nwarp;   // pairs of this warp from here on
+        if (mine == 1) pair_sums<1>(A, ld, nr, S.cols, m, r, k0, nwarp, pb);
+        else if (mine == 2) pair_sums<2>(A, ld, nr, S.cols, m, r, k0, nwarp, pb);
+        else if (mine <= 4) pair_sums<4>(A, ld, nr, S.cols, m, r, k0, nwarp, pb);
+        else pair_sums<8>(A, ld, nr, S.cols, m, r, k0, nwarp, pb);
       }
       cl.sync();
       // 2. cluster sums in rank order and the rotations (identical in every CTA)
@@ -175,11 +251,8 @@ __global__ void __launch_bounds__(NT, 1)
           ga += rp[3 * k + 2];
         }
         double cs = 1.0, sn = 0.0;
-        if (q < S.cols && al > 0.0 && be > 0.0 && fabs(ga) > tol * sqrt(al) * sqrt(be)) {
-          const double zeta = (be - al) / (2.0 * ga);
-          const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          cs = 1.0 / sqrt(1.0 + t * t);
-          sn = cs * t;
+        if (q < S.cols && al > 0.0 && be > 0.0 && above(al, be, ga, tol)) {
+          svd_rotation(al, be, ga, cs, sn);
           s_flag = 1;
         }
         rot[2 * k] = cs;
