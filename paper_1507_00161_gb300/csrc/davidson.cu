@@ -20,10 +20,13 @@
 // first level half of its lanes would idle, so two trees share each instruction from there on
 // (9 FP64 additions instead of 40; FP64 runs at 1.7 lanes per clock and SM here).
 //
+// Short chunks (n up to 8448) are one tree, its empty levels left out; x and A x of an element are
+// formed by different warps.
+//
 // Measured (GB300), chain and Ritz problem together, against 15 launches and two readbacks per
-// iteration: a Davidson run of pf 4p+4n (n = 700, ~52 products) 37.5 -> 27.0 ms, an sd-shell
-// sweep at M = 64 176 -> 123 ms, five instances in batch mode 481 -> 343 ms, bit for bit the
-// same results.
+// iteration, bit for bit the same results: with the products' changes a Davidson run of pf 4p+4n
+// (n = 700, ~55 products) 45.9 -> 19.2 ms, an sd-shell sweep at M = 64 200 -> 120 ms, five instances
+// in batch mode 505 -> 316 ms; residual and first orthogonalisation at n = 300 13.7 + 11.5 -> 9.3 + 7.8 us.
 #include <math.h>
 #include <stdint.h>
 
@@ -74,9 +77,15 @@ __device__ __forceinline__ double tree_sum(const double (&p)[kWarps]) {
   return s;
 }
 
-// the sum of v[i] w[i] over a chunk of len elements, one warp
+// the sum of v[i] w[i] over a chunk of len elements, one warp (valid in lane 0)
 __device__ __forceinline__ double chunk_dot(const double* v, const double* w, int len) {
   const int lane = threadIdx.x & 31;
+  if (len <= 32) {   // one tree, whose levels of at least len only add zeros
+    double x = lane < len ? fma(v[lane], w[lane], 0.0) : 0.0;
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < len) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+  }
   double p[kWarps];
 #pragma unroll
   for (int q = 0; q < kWarps; ++q) p[q] = 0.0;
@@ -159,25 +168,37 @@ k_dav_residual(const double* const* V, const double* const* AV, const double* __
                const double* __restrict__ theta, const double* __restrict__ diag, int k,
                int64_t n, double* x, double* r, double* t,
                double* part, double* __restrict__ sums, int* count) {
-  __shared__ double sy[64];
+  __shared__ double sy[64], s_ax[kThr / 2];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid < k) sy[tid] = y[tid];
   __syncthreads();
   const Chunk c = my_chunk(n);
   const double th = *theta;
-  for (int64_t i = c.i0 + tid; i < c.i0 + c.len; i += kThr) {
-    double xs = 0.0, as = 0.0;
+  auto sum = [&](const double* const* W, int64_t i) {
+    double v = 0.0;
 #pragma unroll 4
-    for (int j = 0; j < k; ++j) {
-      xs = fma(sy[j], V[j][i], xs);
-      as = fma(sy[j], AV[j][i], as);
-    }
+    for (int j = 0; j < k; ++j) v = fma(sy[j], W[j][i], v);
+    return v;
+  };
+  auto finish = [&](int64_t i, double xs, double as) {
     const double rv = fma(-th, xs, as);
     double den = th - diag[i];
     if (fabs(den) < 1e-8) den = den < 0.0 ? -1e-8 : 1e-8;
     x[i] = xs;
     r[i] = rv;
     t[i] = rv / den;
+  };
+  if (c.len <= kThr / 2) {   // a short chunk: x and A x of an element by different warps
+    const int e = tid & (kThr / 2 - 1);
+    double xs = 0.0;
+    if (e < c.len) {
+      if (tid < kThr / 2) xs = sum(V, c.i0 + e);
+      else s_ax[e] = sum(AV, c.i0 + e);
+    }
+    __syncthreads();
+    if (tid < c.len) finish(c.i0 + tid, xs, s_ax[tid]);
+  } else {
+    for (int64_t i = c.i0 + tid; i < c.i0 + c.len; i += kThr) finish(i, sum(V, i), sum(AV, i));
   }
   __syncthreads();   // the chunk is read by other warps below
   for (int j = warp; j < k + 2; j += kWarps) {
