@@ -288,6 +288,7 @@ struct dmrg_ctx {
   // pinned host words for the small per-iteration readbacks (a copy into pageable memory
   // goes through a staging buffer of the driver)
   double* h_words = nullptr;
+  cudaEvent_t read_done = nullptr;   // a readback with work issued behind it
   // the FP64 Rayleigh quotient of the mixed path runs on a stream of its own, overlapping
   // the truncation that follows it (which does not need the energy)
   cudaStream_t rq_stream = nullptr;
@@ -311,6 +312,7 @@ struct dmrg_ctx {
       cudaStreamDestroy(rq_stream);
     }
     if (rq_in) cudaEventDestroy(rq_in);
+    if (read_done) cudaEventDestroy(read_done);
     if (rq_out) cudaEventDestroy(rq_out);
     for (auto e : ev) cudaEventDestroy(e);
     if (h_words) cudaFreeHost(h_words);
@@ -1707,6 +1709,14 @@ static void heff_timed(Ctx& c, Super& sb, const double* x, double* y) {
   c.heff_bytes += sb.bytes;
 }
 
+// take the last heff_timed out of the counts: its product was not needed
+static void heff_untimed(Ctx& c, const Super& sb) {
+  c.ev_used -= 2;
+  c.heff_products -= 1;
+  c.heff_flops -= sb.flops;
+  c.heff_bytes -= sb.bytes;
+}
+
 static double resolve_heff_timing(Ctx& c) {
   sync(c);
   for (int i = 0; i + 1 < c.ev_used; i += 2) {
@@ -1835,6 +1845,7 @@ struct DavRun {
   int nroots = 1;                    // 2: the two lowest states
   const double* guess1 = nullptr;    // second guess, enters the subspace first
   double* out1 = nullptr;            // second state's vector
+  bool ahead = false;                // the pending product has been issued already
 };
 
 static const int kHist = 8;
@@ -1854,11 +1865,22 @@ struct DavPtrs {
   }
 };
 
-static void dav_readback(Ctx& c, const double* d, int cnt, double* h) {
+// `meanwhile` issues work that the host does not wait for here (nullptr: none)
+static void dav_readback(Ctx& c, const double* d, int cnt, double* h,
+                         const std::function<void()>& meanwhile = nullptr) {
   if (!c.h_words) DMRG_CUDA(cudaMallocHost(&c.h_words, sizeof(double) * 64));
-  DMRG_REQUIRE(cnt <= 64, DMRG_EINVAL, "internal: readback too long");
+  DMRG_REQUIRE(cnt <= 32, DMRG_EINVAL, "internal: readback too long");
   DMRG_CUDA(cudaMemcpyAsync(c.h_words, d, sizeof(double) * cnt, cudaMemcpyDeviceToHost, c.stream));
-  sync(c);
+  if (meanwhile) {
+    if (!c.read_done) DMRG_CUDA(cudaEventCreateWithFlags(&c.read_done, cudaEventDisableTiming));
+    DMRG_CUDA(cudaEventRecord(c.read_done, c.stream));
+    meanwhile();
+    const double t0 = wall();
+    DMRG_CUDA(cudaEventSynchronize(c.read_done));
+    c.t_sync += wall() - t0;
+  } else {
+    sync(c);
+  }
   for (int i = 0; i < cnt; ++i) h[i] = c.h_words[i];
 }
 static void dav_d2d(Ctx& c, double* dst, const double* src, int64_t n) {
@@ -1950,8 +1972,16 @@ static void dav_history(Ctx& c, DavRun& R) {
   ++R.nhist;
 }
 
-// consume the product of vector k (py = H v_k), then either finish or request the next
-static void dav_after_product(Ctx& c, DavRun& R) {
+// Products up to this many flops are issued before the host has seen whether the run goes on: the
+// GPU otherwise waits ~25 us for the readback, the host and the launch.  A run that ends leaves
+// one product unused; at the rates of the tile kernels on small superblocks 2e7 flops are 20 to
+// 40 us, which the first iteration or two already save.  Measured (GB300): Davidson run of pf 4p+4n
+// (50 products) 14.5 -> 13.7 ms, sd sweep at M = 64 87 -> 85 ms with the shorter reductions.
+constexpr double kAheadFlops = 2e7;
+
+// consume the product of vector k (py = H v_k), then either finish or request the next (ahead:
+// the next product may be issued at once, R.ahead says so)
+static void dav_after_product(Ctx& c, DavRun& R, bool ahead = false) {
   Super& sb = *R.sb;
   cudaStream_t s = c.stream;
   DavPtrs P(c, R.sub);
@@ -1966,7 +1996,11 @@ static void dav_after_product(Ctx& c, DavRun& R) {
     ++R.nprod;
     dav_chain(DavChain{P.Vp, P.AVp, R.k, n, avec(j), sb.diag.p, P.Hs, 64, P.w, P.Y, c.x.p, c.r.p,
                        c.t.p, vec(R.k), P.sc, P.part, c.dav_count.p}, s);
-    dav_readback(c, P.sc, 4, h);
+    ahead = ahead && sb.flops <= kAheadFlops && R.nprod < c.opt.dav_max_iter;
+    if (ahead)
+      dav_readback(c, P.sc, 4, h, [&] { heff_timed(c, sb, vec(R.k), avec(R.k)); });
+    else
+      dav_readback(c, P.sc, 4, h);
     R.res.theta = h[0];
     R.res.resid = std::sqrt(std::max(h[1], 0.0));
     R.res.nprod = R.nprod;
@@ -1975,11 +2009,13 @@ static void dav_after_product(Ctx& c, DavRun& R) {
     R.res.converged = R.res.resid <= dav_tolerance(c, R.res.theta);
     if (R.res.converged || R.nprod >= c.opt.dav_max_iter ||
         tn <= 1e-14 * std::max(tn0, 1e-300)) {   // (or no new direction left)
+      if (ahead) heff_untimed(c, sb);
       dav_finish(c, R);
       return;
     }
     R.px = vec(R.k);
     R.py = avec(R.k);
+    R.ahead = ahead;
     return;
   }
   multidot(P.Vp, R.k + 1, avec(R.k), n, P.Hs + 64 * R.k, P.part, c.dav_count.p, s);
@@ -2126,9 +2162,10 @@ static DavResult davidson(Ctx& c, Super& sb, const double* guess, double* out,
   dav_begin(c, sb, guess, out, R, guess1, out1);
   while (!R.done) {
     double t0 = wall();
-    heff_timed(c, sb, R.px, R.py);
+    if (!R.ahead) heff_timed(c, sb, R.px, R.py);
+    R.ahead = false;
     const double t1 = wall(), s0 = c.t_sync;
-    dav_after_product(c, R);
+    dav_after_product(c, R, true);
     c.t_detail[16] += t1 - t0;
     c.t_detail[17] += wall() - t1 - (c.t_sync - s0);
     c.t_detail[18] += c.t_sync - s0;
