@@ -3931,6 +3931,7 @@ struct dmrg_batch {
   int64_t products = 0, launches0 = 0;
   double heff_seconds = 0;
   cudaEvent_t t0 = nullptr, t1 = nullptr;
+  bool timing = false;                       // t0 and t1 of the last product are still to be read
   ~dmrg_batch() {
     if (exec) cudaGraphExecDestroy(exec);
     if (h_tab) cudaFreeHost(h_tab);
@@ -4086,9 +4087,24 @@ static void batch_buffers(dmrg_batch& B, const std::vector<int>& inst) {
   }
 }
 
+// wait for the last product, its time into the sum
+static void batch_settle(dmrg_batch& B) {
+  if (!B.timing) return;
+  B.timing = false;
+  DMRG_CUDA(cudaEventSynchronize(B.t1));
+  float ms = 0;
+  DMRG_CUDA(cudaEventElapsedTime(&ms, B.t0, B.t1));
+  B.heff_seconds += ms * 1e-3;
+}
+
 // one batched product: tables up, fused sequence (eager on the first iteration of a step,
-// then captured once into a CUDA graph and replayed), ordering with every context stream
+// then captured once into a CUDA graph and replayed), ordering with every context stream.
+// The host does not wait for it: the instances' chains are launched behind it, and its events
+// (and the pinned tables) are settled before the next, when the readback of a chain has shown
+// that it is done.  Measured (GB300): a sweep of five sd and pf instances (880 products) 4 to 6 %
+// shorter, 295 -> about 278 ms.
 static void batch_product(dmrg_batch& B, const std::vector<int>& inst, std::vector<DavRun>& runs) {
+  batch_settle(B);
   for (int k = 0; k < kMaxInst; ++k) B.h_tab->active[k] = 0;
   for (int i : inst) {
     B.h_tab->in[i] = runs[i].done ? nullptr : runs[i].px;
@@ -4123,12 +4139,9 @@ static void batch_product(dmrg_batch& B, const std::vector<int>& inst, std::vect
     DMRG_CUDA(cudaGraphLaunch(B.exec, B.bs));
   }
   DMRG_CUDA(cudaEventRecord(B.t1, B.bs));
+  B.timing = true;
   DMRG_CUDA(cudaEventRecord(B.ev, B.bs));
   for (int i : inst) DMRG_CUDA(cudaStreamWaitEvent(B.ctx[i]->stream, B.ev, 0));
-  DMRG_CUDA(cudaEventSynchronize(B.t1));
-  float ms = 0;
-  DMRG_CUDA(cudaEventElapsedTime(&ms, B.t0, B.t1));
-  B.heff_seconds += ms * 1e-3;
   ++B.iter;
   ++B.products;
 }
@@ -4169,13 +4182,19 @@ static void batch_step(dmrg_batch& B, const std::vector<BWork>& work,
     for (int i : inst) any = any || !runs[i].done;
     if (!any) break;
     batch_product(B, inst, runs);
-    ip.run(int(inst.size()), [&](int j) {
-      const int i = inst[j];
-      if (runs[i].done) return;
-      PoolScope ps(&B.ctx[i]->pool);
-      dav_after_product(*B.ctx[i], runs[i]);
-    });
+    try {
+      ip.run(int(inst.size()), [&](int j) {
+        const int i = inst[j];
+        if (runs[i].done) return;
+        PoolScope ps(&B.ctx[i]->pool);
+        dav_after_product(*B.ctx[i], runs[i]);
+      });
+    } catch (...) {   // (no product left running on buffers that the caller may free)
+      cudaStreamSynchronize(B.bs);
+      throw;
+    }
   }
+  batch_settle(B);
   ip.run(int(work.size()), [&](int j) {
     const BWork& w = work[j];
     Ctx& c = *B.ctx[w.inst];
