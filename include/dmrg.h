@@ -443,8 +443,8 @@ int dmrg_heff_cost(dmrg_ctx* ctx, int32_t p, double* flops, double* bytes, int64
  * contexts (1..64, same precision, blocks built).  dmrg_batch_sweep runs one sweep of
  * every context in lockstep: at step j each context does its own j-th two-site step
  * (position order as in dmrg_sweep; contexts with fewer steps drop out), and every
- * Davidson iteration computes the H_eff products of all contexts still iterating in ONE
- * fused kernel launch (tiles of all superblocks in one list), recorded once per step in a
+ * Davidson iteration computes the H_eff products of all contexts still iterating in the
+ * same kernel launches (tiles of all superblocks in one list), recorded once per step in a
  * CUDA graph on an internal stream and replayed with new vector pointers.  Each context's
  * own work (superblock, prediction, the host side of its Davidson iterations, truncation)
  * runs on a host thread of its own and on the context's stream, so contexts created with
