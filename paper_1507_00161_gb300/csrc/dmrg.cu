@@ -1763,6 +1763,8 @@ __global__ void k_set_hs_diag(double* H, int ld, const double* w) {
   }
 }
 
+static const int kMaxSub = 64;   // most subspace vectors
+
 static void ensure_ws(Ctx& c, int64_t n, int sub) {
   if (c.ws_n >= n && c.ws_sub >= sub) return;
   int64_t nn = std::max<int64_t>(n, 1);
@@ -1779,10 +1781,11 @@ static void ensure_ws(Ctx& c, int64_t n, int sub) {
   c.partials.alloc(66 * 300);
   c.dav_count.alloc(1);
   DMRG_CUDA(cudaMemsetAsync(c.dav_count.p, 0, sizeof(int), c.stream));
-  std::vector<const double*> ptrs(2 * sub);
+  // the vectors V, then from kMaxSub on A V: a later run with another `sub` finds both
+  std::vector<const double*> ptrs(2 * kMaxSub, nullptr);
   for (int j = 0; j < sub; ++j) {
     ptrs[j] = c.V.p + j * nn;
-    ptrs[sub + j] = c.AV.p + j * nn;
+    ptrs[kMaxSub + j] = c.AV.p + j * nn;
   }
   c.vptr.upload(ptrs, c.stream);
   c.ws_n = nn;
@@ -1854,14 +1857,14 @@ struct DavPtrs {
   double *Hs, *w, *Y, *sc, *part;
   const double* const* Vp;
   const double* const* AVp;
-  DavPtrs(Ctx& c, int sub) {
+  explicit DavPtrs(Ctx& c) {
     Hs = c.small.p;              // 64 x 64, row k holds <v_i, H v_k>, i <= k
     w = Hs + 64 * 64;            // Ritz values, ascending
     Y = w + 64;                  // rows 0 and 1 = coefficients of the two lowest Ritz vectors
     sc = Y + 64 * 64;            // device scalars
     part = c.partials.p;
     Vp = c.vptr.p;
-    AVp = c.vptr.p + sub;
+    AVp = c.vptr.p + kMaxSub;
   }
 };
 
@@ -1895,7 +1898,7 @@ static void dav_begin(Ctx& c, Super& sb, const double* guess, double* out, DavRu
   R.nroots = out1 ? 2 : 1;
   R.guess1 = guess1;
   R.out1 = out1;
-  R.sub = std::max(4, std::min(64, c.opt.dav_max_sub));
+  R.sub = std::max(4, std::min(kMaxSub, c.opt.dav_max_sub));
   R.out = out;
   ensure_ws(c, R.n, R.sub);
   ensure_diag(c, sb);
@@ -1908,7 +1911,7 @@ static void dav_begin(Ctx& c, Super& sb, const double* guess, double* out, DavRu
     c.hist_tmp.alloc(R.ld);
   }
   c.mlp_sc.alloc(64);
-  DavPtrs P(c, R.sub);
+  DavPtrs P(c);
   double* v0 = c.V.p;
   dav_d2d(c, v0, guess, R.n);
   dot(v0, v0, R.n, P.sc, P.part, c.stream);
@@ -1919,7 +1922,7 @@ static void dav_begin(Ctx& c, Super& sb, const double* guess, double* out, DavRu
 
 static void dav_finish(Ctx& c, DavRun& R) {
   Super& sb = *R.sb;
-  DavPtrs P(c, R.sub);
+  DavPtrs P(c);
   const int64_t n = R.n;
   double h[2];
   dot(c.x.p, c.x.p, n, P.sc + 4, P.part, c.stream);
@@ -1964,7 +1967,7 @@ static double dav_tolerance(const Ctx& c, double theta) {
 // iterate, residual and Ritz value for training
 static void dav_history(Ctx& c, DavRun& R) {
   if (!c.mlp_harvest || R.nhist >= kHist) return;
-  DavPtrs P(c, R.sub);
+  DavPtrs P(c);
   dav_d2d(c, c.hist_x.p + R.nhist * R.ld, c.x.p, R.n);
   dav_d2d(c, c.hist_r.p + R.nhist * R.ld, c.r.p, R.n);
   DMRG_CUDA(cudaMemcpyAsync(c.hist_theta.p + R.nhist, P.w, sizeof(double),
@@ -1984,7 +1987,7 @@ constexpr double kAheadFlops = 2e7;
 static void dav_after_product(Ctx& c, DavRun& R, bool ahead = false) {
   Super& sb = *R.sb;
   cudaStream_t s = c.stream;
-  DavPtrs P(c, R.sub);
+  DavPtrs P(c);
   const int64_t n = R.n, ld = R.ld;
   auto vec = [&](int j) { return c.V.p + j * ld; };
   auto avec = [&](int j) { return c.AV.p + j * ld; };
