@@ -1,15 +1,18 @@
-// FP64 division, reciprocal and square root for latency, with the results of the library's, shared by
-// the Jacobi kernels.  One FP64 instruction of a warp takes 64 clocks here whatever follows it, so a
+// FP64 division, reciprocal and square root for latency, shared by the Jacobi kernels (the Ritz problem
+// and the SVD).  One FP64 instruction of a warp takes 64 clocks here whatever follows it, so a
 // dependent operation less is what counts (measured: division 564 -> 364 clocks, root 598 -> 430).
 #pragma once
 #include <cuda_runtime.h>
 
 namespace dmrg {
 
-// Quotient, reciprocal and square root, rounded to nearest, by Newton's iteration with a final
-// correction from the exact remainder (P. Markstein, IBM J. Res. Dev. 34 (1990) 111): from a 2^-23
-// seed one step gives a reciprocal good to 2^-46 and, with the remainder, a result good to ~2^-90
-// before its one rounding.  Operands in 2^-400 .. 2^400.
+// Quotient, reciprocal and square root by Newton's iteration with a final correction from the
+// remainder, formed by a fused multiply-add (P. Markstein, IBM J. Res. Dev. 34 (1990) 111).  The seed
+// instructions read the upper 32 bits of their operand and give the upper 32 bits of a result, so a
+// seed is good to 2^-19 (two cuts at a 20-bit mantissa); one step gives 2^-38, and the correction a
+// value good to 2^-75 before its one rounding.  That rounds to nearest unless the exact value lies
+// within 2^-75 of the middle between two numbers (at most one operand in 2^21); there the result may
+// be the other neighbour, one unit in the last place from the library's.  Operands in 2^-399 .. 2^400.
 __device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 __device__ __forceinline__ bool mid_range(double x) {
   const int e = exponent(x);
