@@ -595,14 +595,22 @@ struct LayDev {
   int32_t pblk0, pblk1, poff1, D;
 };
 // renormalization of one operator block O (enlarged sectors so, si) at xoff -> O' at yoff, columns
-// c0 .. c0 + 31 of O' (renorm.cu).  Blocks come in three classes by size (project_class), each with
-// its units one after the other: units of class k at [begin[k], begin[k + 1])
+// c0 .. c0 + project_cols - 1 of O' (renorm.cu).  Blocks come in three classes by size
+// (project_class), each with its units one after the other: units of class k at [begin[k],
+// begin[k + 1])
 struct ProjTask {
   int64_t xoff, yoff;
   int32_t so, si, c0, pad;
 };
-int project_class(int Do, int Di);
-int project_units(int cls, int mi);
+constexpr int kProjTiny = 16;
+constexpr int project_class(int Do, int Di) {
+  return Do <= kProjTiny && Di <= kProjTiny ? 0 : Do <= 32 ? 1 : 2;
+}
+constexpr int project_cols(int cls) { return cls == 2 ? 8 : 32; }
+constexpr int project_units(int cls, int mi) {
+  return cls == 0 ? 1 : cls == 1 ? (mi + project_cols(1) - 1) / project_cols(1)
+                                 : (mi + project_cols(2) - 1) / project_cols(2);
+}
 void project_blocks(const ProjTask* units, const int64_t (&begin)[4], const int32_t* D,
                     const int32_t* m, const int64_t* uoff, const double* X, const double* U,
                     double* Y, cudaStream_t s);

@@ -887,7 +887,7 @@ static void project(Ctx& c, OpSet& E, const Iso& iso, OpSet& out) {
   out.lab_ptr.assign(E.nlab + 1, 0);
   out.blocks.clear();
   double tp = wall();
-  // one renormalization unit per kept block (and 32 columns of a wide one), built label by label:
+  // one renormalization unit per kept block (and some columns of a wide one), built label by label:
   // counts first, then every label fills its own ranges
   struct Count {
     int64_t blocks = 0, elems = 0, units[3] = {0, 0, 0};
@@ -933,7 +933,7 @@ static void project(Ctx& c, OpSet& E, const Iso& iso, OpSet& out) {
         out.blocks[c0.blocks++] = OpBlock{iso.kept_idx[b.so], iso.kept_idx[b.si], c0.elems};
         const int cls = project_class(Do, Di), nu = project_units(cls, mi);
         for (int u = 0; u < nu; ++u)
-          units[begin[cls] + c0.units[cls]++] = ProjTask{b.off, c0.elems, b.so, b.si, 32 * u, 0};
+          units[begin[cls] + c0.units[cls]++] = ProjTask{b.off, c0.elems, b.so, b.si, project_cols(cls) * u, 0};
         c0.elems += int64_t(iso.m[b.so]) * mi;
       });
     }

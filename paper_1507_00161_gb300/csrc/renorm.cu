@@ -8,13 +8,15 @@
 // time, and nothing is computed for padding; the operands are read where they are (rows of O and
 // columns of U_o broadcast, rows of U_i consecutive).  Driven by the block table itself:
 //  - blocks with D_o, D_i <= 16: one warp each, T in shared memory;
-//  - larger blocks: units of a block and up to 32 columns of U_i, one thread block each, T in
-//    shared memory, 32 or 128 of its rows at a time; with more rows than that the result grows
-//    chunk by chunk in its place.
+//  - larger blocks: units of a block and some columns of U_i, one thread block each, T in shared
+//    memory: 32 columns of blocks of up to 32 rows, 8 columns of taller ones, 128 rows at a time
+//    (with more rows the result grows chunk by chunk in its place).  The tallest block's units are
+//    the tail of the launch, and narrow ones keep that short.
 // FP64 throughout, every sum in index order (deterministic).
 // Measured (GB300) against 32 x 32 tiles in two passes through a scratch and one warp per block up to
-// 32: all right blocks of pf 8p+8n, M0 = 4096, 361 -> 270 ms of kernels; at M = 4096, position 15, the
-// two steps of a pair 1.5 -> 0.5 ms each.
+// 32, kernels of all right blocks: pf 8p+8n, M0 = 4096, 361 -> 249 ms (270 with 32 columns), pf 4p+4n,
+// M0 = 2000, 235 -> 187 ms (270), sd 2p+2n, M0 = 512, 5.3 -> 5.1 ms (11.5), M0 = 128 1.18 -> 0.97 ms
+// (1.35); at M = 4096, position 15, the two steps of a pair 1.5 -> 0.5 ms each.
 #include <stdint.h>
 
 #include "common.h"
@@ -23,10 +25,8 @@ namespace dmrg {
 
 namespace {
 
-constexpr int kCols = 32;            // columns of a unit
-constexpr int kLd = kCols + 1;
 constexpr int kThr = 128;
-constexpr int kTiny = 16, kTinyLd = kTiny + 1;
+constexpr int kTiny = kProjTiny, kTinyLd = kTiny + 1;
 constexpr int kTinyWarps = 4;
 
 // c[r * 1] ... sum_k a[k sa] b[k sb], k < n, in order
@@ -37,15 +37,16 @@ __device__ __forceinline__ double dot_strided(const double* __restrict__ a, int6
   return s;
 }
 
-template <int ROWS>
+template <int ROWS, int COLS>
 __global__ void __launch_bounds__(kThr, ROWS == 32 ? 12 : 6)
 k_project(const ProjTask* __restrict__ units, const int32_t* __restrict__ D,
           const int32_t* __restrict__ m, const int64_t* __restrict__ uoff,
           const double* __restrict__ X, const double* __restrict__ U, double* __restrict__ Y) {
+  constexpr int kLd = COLS + 1;
   __shared__ double T[ROWS * kLd];
   const ProjTask pt = units[blockIdx.x];
   const int Do = D[pt.so], Di = D[pt.si], mo = m[pt.so], mi = m[pt.si];
-  const int n = min(kCols, mi - pt.c0);
+  const int n = min(COLS, mi - pt.c0);
   const double* __restrict__ Xb = X + pt.xoff;
   const double* __restrict__ Ui = U + uoff[pt.si] + pt.c0;
   const double* __restrict__ Uo = U + uoff[pt.so];
@@ -105,21 +106,16 @@ k_project_tiny(const ProjTask* __restrict__ tasks, int64_t n, const int32_t* __r
 
 }  // namespace
 
-int project_class(int Do, int Di) {
-  return Do <= kTiny && Di <= kTiny ? 0 : Do <= 32 ? 1 : 2;
-}
-int project_units(int cls, int mi) { return cls == 0 ? 1 : (mi + kCols - 1) / kCols; }
-
 void project_blocks(const ProjTask* units, const int64_t (&begin)[4], const int32_t* D,
                     const int32_t* m, const int64_t* uoff, const double* X, const double* U,
                     double* Y, cudaStream_t s) {
   const int64_t n0 = begin[1] - begin[0], n1 = begin[2] - begin[1], n2 = begin[3] - begin[2];
   if (n2 > 0) {   // the widest first
-    k_project<128><<<int(n2), kThr, 0, s>>>(units + begin[2], D, m, uoff, X, U, Y);
+    k_project<128, project_cols(2)><<<int(n2), kThr, 0, s>>>(units + begin[2], D, m, uoff, X, U, Y);
     DMRG_LAUNCHED();
   }
   if (n1 > 0) {
-    k_project<32><<<int(n1), kThr, 0, s>>>(units + begin[1], D, m, uoff, X, U, Y);
+    k_project<32, project_cols(1)><<<int(n1), kThr, 0, s>>>(units + begin[1], D, m, uoff, X, U, Y);
     DMRG_LAUNCHED();
   }
   if (n0 > 0) {
