@@ -558,11 +558,11 @@ void heff_reduce_slots(const HeffRed* d_red, int64_t n_plain, int64_t n_red, con
                        cudaStream_t s);
 // mixed path: the same product with 3xTF32 warp MMAs (heff_tc.cu); d_order: the tiles' order by
 // heff_tc_order, whose first n_wide are the wide ones (its return value): wide on s, the
-// narrow ones on s_narrow
+// narrow ones on s_narrow.  Not apart: all tiles in one launch as wide ones
 void heff_tc(const HeffTile* d_tiles, const int32_t* d_order, int64_t n_wide, int64_t n_tiles,
              const HeffItem* d_items, const HeffPtrs<float>& ptrs, cudaStream_t s,
              cudaStream_t s_narrow);
-int64_t heff_tc_order(const std::vector<HeffTile>& tiles, std::vector<int32_t>& order);
+int64_t heff_tc_order(const std::vector<HeffTile>& tiles, bool apart, std::vector<int32_t>& order);
 template <class TO>
 void pad_psi(const double* x, TO* xp, const int64_t* src_off, const int64_t* dst_off,
              const int32_t* len, int nblocks, cudaStream_t s);

@@ -173,6 +173,7 @@ struct Super {
   DevBuf<HeffRed> fred;
   DevBuf<int32_t> forder;            // order of the tiles in the mixed kernel, n_fwide wide ones first
   int64_t n_fwide = 0;
+  bool beside = false;   // tiles_beside
   // sums of partial tiles (n_plain: small-block tiles, first in the list); elements of the
   // partial tiles of the small-block kernel and of the tile kernels, one after the other
   int64_t n_ftiles = 0, n_stiles = 0, n_fred = 0, n_plain = 0, p_elems = 0, q_elems = 0;
@@ -1021,6 +1022,19 @@ static OpSet vacuum_ops(int nlab, int which, cudaStream_t s) {
   return v;
 }
 
+// Whether the mixed kernels of a product run side by side (tile_kernels), the wide and the narrow tiles
+// as launches of their own; otherwise one after the other, with one launch for all tiles.  Two
+// streams cost host calls in an eager product and 10 to 40 us in the capture at the second one, which
+// every new superblock pays.  Beside grouped passes a few tiles repay that: measured (GB300; repeated
+// product, second product), pf 4p+4n at position 4 (18 tiles) 213 -> 198 us and 314 -> 325, pf 8p+8n at
+// position 5 (33 tiles) 430 -> 393 and 532 -> 532, but three tiles 163 -> 162 and 266 -> 288.  Tiles
+// alone fill the chip from ~270 on (seven units per SM, four a tile): 296 tiles 100 -> 87 us with ONE
+// launch, 759 tiles 160 -> 155 and 252 -> 284 with two streams (even after ten products), 1309 tiles
+// 205 -> 196 and 309 -> 330, 4003 tiles 803 -> 723 and 898 -> 862.
+static bool tiles_beside(int64_t n_tiles, bool any_big) {
+  return n_tiles >= (any_big ? 4 : 1024);
+}
+
 // ---------------------------------------------------------------------------------------
 // superblock at position p: enlarged operators, wave-function layout, H_eff task lists
 // ---------------------------------------------------------------------------------------
@@ -1301,7 +1315,10 @@ static void build_super(Ctx& c, int p) {
     sb->fitems.upload(fi, c.stream);
     sb->ftiles.upload(tl, c.stream);
     std::vector<int32_t> order;
-    sb->n_fwide = heff_tc_order(tl, order);
+    const bool any_big = std::find(big_bo.begin(), big_bo.end(), 1) != big_bo.end();
+    sb->beside = tiles_beside(int64_t(tl.size()), any_big);
+    if (sb->beside || (any_big && !tl.empty())) c.side.create();   // (70 us: not in the first product)
+    sb->n_fwide = heff_tc_order(tl, sb->beside, order);
     sb->forder.upload(order, c.stream);
     sb->stiles.upload(tls, c.stream);
     sb->fred.upload(fr, c.stream);
@@ -1518,36 +1535,40 @@ static void heff_buffers(Ctx& c, Super& sb, int prec) {
 }
 
 // The kernels of the output blocks of one precision on main stream st: small blocks, tiles, and
-// the two grouped passes of the big blocks (`big`, writing to their own blocks).  They do not
-// depend on each other, and each alone leaves the chip partly idle (its last wave; a few large
-// tasks), so they run side by side: the grouped passes, or else the wide tiles, on st, the rest
-// on the side stream; then the partial tiles are added.  Measured (GB300): pf 4p+4n at
-// position 6 (five short kernels) 136 -> 89 us per product, the mixed one of pf 4p+5n 83 -> 78 us.
+// the two grouped passes of the big blocks (`big`, writing to their own blocks); then the partial
+// tiles are added.  The kernels do not depend on each other, and each alone leaves the chip partly idle
+// (its last wave; a few large tasks), so with enough work they run side by side:
+// the grouped passes, or else the wide tiles, on st, the rest on the side stream.
 struct TileLists {
   const HeffTile *stiles, *tiles;
   const int32_t* order;
   const HeffItem* items;
   const HeffRed* red;
   int64_t n_stiles, n_tiles, n_wide, n_plain, n_red;
+  bool beside;   // tiles_beside: wide and narrow tiles apart, the kernels side by side
 };
+
 template <class F>
 static void tile_kernels(const TileLists& l, const HeffPtrs<double>& p, SideStream& side,
                          cudaStream_t st, bool any_big, F&& big) {
-  cudaStream_t sd = side.begin(st);
+  // the tiles beside the grouped passes (few long chains each): pf 8p+8n at position 5 353 -> 229 us,
+  // sd 4p+4n at position 4 (two tiles) 153 -> 140; the small blocks alone are not worth a second stream
+  const bool fork = any_big && l.n_tiles > 0;
+  cudaStream_t sd = fork ? side.begin(st) : st;
   heff_small<double>(l.stiles, l.n_stiles, l.items, p, sd);
-  heff_fused64(l.tiles, l.n_tiles, l.items, p, any_big ? sd : st);
+  heff_fused64(l.tiles, l.n_tiles, l.items, p, sd);
   if (any_big) big();
-  side.end(st);
+  if (fork) side.end(st);
   heff_reduce_slots<double>(l.red, l.n_plain, l.n_red, p, st);
 }
 template <class F>
 static void tile_kernels(const TileLists& l, const HeffPtrs<float>& p, SideStream& side,
                          cudaStream_t st, bool any_big, F&& big) {
-  cudaStream_t sd = side.begin(st);
+  cudaStream_t sd = l.beside ? side.begin(st) : st;
   heff_small<float>(l.stiles, l.n_stiles, l.items, p, sd);
   heff_tc(l.tiles, l.order, l.n_wide, l.n_tiles, l.items, p, any_big ? sd : st, sd);
   if (any_big) big();
-  side.end(st);
+  if (l.beside) side.end(st);
   heff_reduce_slots<float>(l.red, l.n_plain, l.n_red, p, st);
 }
 
@@ -1591,7 +1612,7 @@ static void big_passes(Ctx& c, Super& sb, float* y, const int32_t* active, cudaS
 // is needed.
 static void heff_core(Ctx& c, Super& sb, int prec, double* y64, cudaStream_t st) {
   const TileLists l{sb.stiles.p, sb.ftiles.p, sb.forder.p, sb.fitems.p, sb.fred.p, sb.n_stiles,
-                    sb.n_ftiles, sb.n_fwide, sb.n_plain, sb.n_fred};
+                    sb.n_ftiles, sb.n_fwide, sb.n_plain, sb.n_fred, sb.beside};
   const bool big = sb.n_big_blocks > 0;
   if (prec == 0) {
     HeffPtrs<double> ptr{};
@@ -3929,6 +3950,7 @@ struct dmrg_batch {
   dmrg::DevBuf<int32_t> order;
   int64_t n_wide = 0;
   int64_t n_tiles = 0, n_stiles = 0, n_red = 0, n_plain = 0;
+  bool beside = false, any_big = false;      // tiles_beside; some superblock has grouped passes
   // per-iteration tables: input and output vector pointers, active flags
   struct Tab {
     const double* in[dmrg::kMaxInst];
@@ -4002,7 +4024,10 @@ static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
   B.items.upload(fi, B.bs);
   B.tiles.upload(tl, B.bs);
   std::vector<int32_t> order;
-  B.n_wide = heff_tc_order(tl, order);
+  B.any_big = false;
+  for (int i : inst) B.any_big = B.any_big || B.ctx[i]->sb->n_big_blocks > 0;
+  B.beside = tiles_beside(int64_t(tl.size()), B.any_big);
+  B.n_wide = heff_tc_order(tl, B.beside, order);
   B.order.upload(order, B.bs);
   B.stiles.upload(tls, B.bs);
   B.n_plain = int64_t(fr.size());
@@ -4019,9 +4044,8 @@ static void batch_lists(dmrg_batch& B, const std::vector<int>& inst) {
 static void batch_issue(dmrg_batch& B, const std::vector<int>& inst) {
   const int32_t* act = B.d_tab->active;
   const TileLists l{B.stiles.p, B.tiles.p, B.order.p, B.items.p, B.red.p, B.n_stiles,
-                    B.n_tiles, B.n_wide, B.n_plain, B.n_red};
-  bool any_big = false;
-  for (int i : inst) any_big = any_big || B.ctx[i]->sb->n_big_blocks > 0;
+                    B.n_tiles, B.n_wide, B.n_plain, B.n_red, B.beside};
+  const bool any_big = B.any_big;
   if (B.precision == DMRG_FP64) {
     HeffPtrs<double> ptr{};
     ptr.active = act;

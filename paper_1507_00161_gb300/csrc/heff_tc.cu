@@ -289,12 +289,13 @@ void heff_tc(const HeffTile* d_tiles, const int32_t* d_order, int64_t n_wide, in
   }
 }
 
-int64_t heff_tc_order(const std::vector<HeffTile>& tiles, std::vector<int32_t>& order) {
+int64_t heff_tc_order(const std::vector<HeffTile>& tiles, bool apart, std::vector<int32_t>& order) {
   order.clear();
   order.reserve(tiles.size());
   for (size_t i = 0; i < tiles.size(); ++i)
-    if (tiles[i].n > tc::kNarrow) order.push_back(int32_t(i));
+    if (!apart || tiles[i].n > tc::kNarrow) order.push_back(int32_t(i));
   const int64_t n_wide = int64_t(order.size());
+  if (!apart) return n_wide;
   for (size_t i = 0; i < tiles.size(); ++i)
     if (tiles[i].n <= tc::kNarrow) order.push_back(int32_t(i));
   return n_wide;
