@@ -9,7 +9,8 @@
 //    iteration: davidson.cu).
 //  * symmetric eigensolver: parallel-ordered cyclic Jacobi (jacobi.cuh), one thread block per
 //    matrix, FP64 (density matrices of sectors too wide for the cluster SVD).
-//  * selection of the M-th largest weight (bitonic sort in one block) and kept counts.
+//  * selection of the M-th largest weight (radix selection; for DBSS a bitonic sort in one block)
+//    and kept counts.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -284,8 +285,6 @@ void run_gemm_tasks(const DevTaskList& L, const Bases<T>& b, int beta_zero, cuda
 }
 template void run_gemm_tasks<double>(const DevTaskList&, const Bases<double>&, int, cudaStream_t,
                                      const int32_t*);
-template void run_gemm_tasks<float>(const DevTaskList&, const Bases<float>&, int, cudaStream_t,
-                                    const int32_t*);
 
 // ------------------------------------------------------------------------------------
 // copy tasks (one warp per destination sub-block)

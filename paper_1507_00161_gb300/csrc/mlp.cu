@@ -27,7 +27,6 @@ int64_t mlp_n_params() {
   return int64_t(kWd) * kIn + kWd + 2 * (int64_t(kWd) * kWd + kWd) + kWd + 1;
 }
 
-template <class T>
 struct MlpOffsets {
   int64_t W1, b1, W2, b2, W3, b3, w4, b4;
   MlpOffsets() {
@@ -43,41 +42,38 @@ struct MlpOffsets {
 };
 
 // ------------------------------------------------------------------------------------
-// elementwise kernels
+// elementwise kernels (the first four: FP64 network only)
 // ------------------------------------------------------------------------------------
-template <class T>
-__global__ void k_bias_relu(T* __restrict__ Z, const T* __restrict__ b, T* __restrict__ H,
-                            int64_t rows, int cols) {
+__global__ void k_bias_relu(double* __restrict__ Z, const double* __restrict__ b,
+                            double* __restrict__ H, int64_t rows, int cols) {
   const int64_t n = rows * cols;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
-    const T z = Z[i] + b[i % cols];
+    const double z = Z[i] + b[i % cols];
     Z[i] = z;
-    H[i] = z > T(0) ? z : T(0);
+    H[i] = z > 0.0 ? z : 0.0;
   }
 }
 
-template <class T>
-__global__ void k_add_scalar(T* __restrict__ y, const T* __restrict__ b, int64_t n) {
+__global__ void k_add_scalar(double* __restrict__ y, const double* __restrict__ b, int64_t n) {
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x)
     y[i] += b[0];
 }
 
 // dZ = dH * (Z > 0)
-template <class T>
-__global__ void k_relu_grad(const T* __restrict__ Z, T* __restrict__ dH, int64_t n) {
+__global__ void k_relu_grad(const double* __restrict__ Z, double* __restrict__ dH, int64_t n) {
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x)
-    if (!(Z[i] > T(0))) dH[i] = T(0);
+    if (!(Z[i] > 0.0)) dH[i] = 0.0;
 }
 
 // column sums of a rows x cols matrix (one thread per column, fixed order)
-template <class T>
-__global__ void k_colsum(const T* __restrict__ A, int64_t rows, int cols, T* __restrict__ out) {
+__global__ void k_colsum(const double* __restrict__ A, int64_t rows, int cols,
+                         double* __restrict__ out) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= cols) return;
-  T s = T(0);
+  double s = 0.0;
   for (int64_t r = 0; r < rows; ++r) s += A[r * cols + c];
   out[c] = s;
 }
@@ -213,9 +209,8 @@ static int grid_for(int64_t n) {
 
 // C (M x N, ldc) = op(A) op(B) through the task-list GEMM; sizes of the three buffers in
 // elements for the host-side range check
-template <class T>
-static void gemm(T* C, int ldc, const T* A, int lda, bool ta, const T* B, int ldb, bool tb, int M,
-                 int N, int K, int64_t nA, int64_t nB, int64_t nC, cudaStream_t s) {
+static void gemm(double* C, int ldc, const double* A, int lda, bool ta, const double* B, int ldb,
+                 bool tb, int M, int N, int K, int64_t nA, int64_t nB, int64_t nC, cudaStream_t s) {
   TaskList L;
   L.begin_task(Operand{0, B_Y, ldc}, M, N);
   L.add_term(Operand{0, B_X, lda}, Operand{0, B_U, ldb}, K, (ta ? 1 : 0) | (tb ? 2 : 0), 1.0);
@@ -225,11 +220,11 @@ static void gemm(T* C, int ldc, const T* A, int lda, bool ta, const T* B, int ld
   be[B_Y] = nC;
   DevTaskList d;
   d.build(L, be, s);
-  Bases<T> b{};
-  b.p[B_X] = const_cast<T*>(A);
-  b.p[B_U] = const_cast<T*>(B);
+  Bases<double> b{};
+  b.p[B_X] = const_cast<double*>(A);
+  b.p[B_U] = const_cast<double*>(B);
   b.p[B_Y] = C;
-  run_gemm_tasks<T>(d, b, 1, s);
+  run_gemm_tasks<double>(d, b, 1, s);
   DMRG_CUDA(cudaStreamSynchronize(s));   // the list buffers are released on return
 }
 
@@ -238,7 +233,8 @@ static void gemm(T* C, int ldc, const T* A, int lda, bool ta, const T* B, int ld
 // ------------------------------------------------------------------------------------
 constexpr int kRows = 64;   // samples of one part of a sum over the minibatch
 
-// y = H3 w4 + b4: one warp per sample, compensated sums
+// y = H3 w4 + b4: one warp per sample, a compensated sum of eight products per lane, then a plain tree
+// over the lanes
 __global__ void __launch_bounds__(256) k_output(const float* __restrict__ H,
                                                 const float* __restrict__ w,
                                                 const float* __restrict__ b, int64_t B,
@@ -335,7 +331,7 @@ static void add_parts(const float* p, int parts, int64_t stride, int64_t n, floa
 }
 
 static void forward32(const float* P, const float* X, int64_t B, MlpActs<float>& a, cudaStream_t s) {
-  MlpOffsets<float> o;
+  MlpOffsets o;
   auto layer = [&](const float* in, int n_in, int64_t W, int64_t b, float* out) {
     dense_gemm_tc(DenseGemm{in, P + W, out, P + b, int(B), kWd, n_in, n_in, n_in, kWd, 2, n_in, 0},
                   DenseEpilogue::bias_relu, 1, s);
@@ -350,7 +346,7 @@ static void forward32(const float* P, const float* X, int64_t B, MlpActs<float>&
 // gradients from a.dY on
 static void backward32(const float* P, const float* X, int64_t B, MlpActs<float>& a, float* G,
                        cudaStream_t s) {
-  MlpOffsets<float> o;
+  MlpOffsets o;
   const int parts = int((B + kRows - 1) / kRows);
   // a weight gradient in parts of at least 128 samples, two thread blocks per SM at most
   const int splits = int(std::max<int64_t>(1, std::min<int64_t>(19, (B + 127) / 128)));
@@ -380,31 +376,32 @@ static void backward32(const float* P, const float* X, int64_t B, MlpActs<float>
   add_parts(a.sums.p + kWd, parts, 5 * kWd, kWd * kIn, G + o.W1, s);
 }
 
+static void forward64(const double* P, const double* X, int64_t B, MlpActs<double>& a, cudaStream_t s) {
+  MlpOffsets o;
+  const int64_t np = mlp_n_params();
+  const int64_t nh = B * kWd;
+  gemm(a.Z1.p, kWd, X, kIn, false, P + o.W1, kIn, true, int(B), kWd, kIn, B * kIn, np - o.W1,
+          nh, s);
+  k_bias_relu<<<grid_for(nh), 256, 0, s>>>(a.Z1.p, P + o.b1, a.H1.p, B, kWd);
+  DMRG_LAUNCHED();
+  gemm(a.Z2.p, kWd, a.H1.p, kWd, false, P + o.W2, kWd, true, int(B), kWd, kWd, nh, np - o.W2,
+          nh, s);
+  k_bias_relu<<<grid_for(nh), 256, 0, s>>>(a.Z2.p, P + o.b2, a.H2.p, B, kWd);
+  DMRG_LAUNCHED();
+  gemm(a.Z3.p, kWd, a.H2.p, kWd, false, P + o.W3, kWd, true, int(B), kWd, kWd, nh, np - o.W3,
+          nh, s);
+  k_bias_relu<<<grid_for(nh), 256, 0, s>>>(a.Z3.p, P + o.b3, a.H3.p, B, kWd);
+  DMRG_LAUNCHED();
+  gemm(a.Y.p, 1, a.H3.p, kWd, false, P + o.w4, kWd, true, int(B), 1, kWd, nh, np - o.w4, B, s);
+  k_add_scalar<<<grid_for(B), 256, 0, s>>>(a.Y.p, P + o.b4, B);
+  DMRG_LAUNCHED();
+}
+
 template <class T>
 void mlp_forward(const T* P, const T* X, int64_t B, MlpActs<T>& a, cudaStream_t s) {
-  MlpOffsets<T> o;
-  const int64_t np = mlp_n_params();
   a.ensure(B);
-  const int64_t nh = B * kWd;
-  if constexpr (std::is_same<T, float>::value) {
-    forward32(P, X, B, a, s);
-    return;
-  }
-  gemm<T>(a.Z1.p, kWd, X, kIn, false, P + o.W1, kIn, true, int(B), kWd, kIn, B * kIn, np - o.W1,
-          nh, s);
-  k_bias_relu<T><<<grid_for(nh), 256, 0, s>>>(a.Z1.p, P + o.b1, a.H1.p, B, kWd);
-  DMRG_LAUNCHED();
-  gemm<T>(a.Z2.p, kWd, a.H1.p, kWd, false, P + o.W2, kWd, true, int(B), kWd, kWd, nh, np - o.W2,
-          nh, s);
-  k_bias_relu<T><<<grid_for(nh), 256, 0, s>>>(a.Z2.p, P + o.b2, a.H2.p, B, kWd);
-  DMRG_LAUNCHED();
-  gemm<T>(a.Z3.p, kWd, a.H2.p, kWd, false, P + o.W3, kWd, true, int(B), kWd, kWd, nh, np - o.W3,
-          nh, s);
-  k_bias_relu<T><<<grid_for(nh), 256, 0, s>>>(a.Z3.p, P + o.b3, a.H3.p, B, kWd);
-  DMRG_LAUNCHED();
-  gemm<T>(a.Y.p, 1, a.H3.p, kWd, false, P + o.w4, kWd, true, int(B), 1, kWd, nh, np - o.w4, B, s);
-  k_add_scalar<T><<<grid_for(B), 256, 0, s>>>(a.Y.p, P + o.b4, B);
-  DMRG_LAUNCHED();
+  if constexpr (std::is_same<T, float>::value) forward32(P, X, B, a, s);
+  else forward64(P, X, B, a, s);
 }
 
 static double mlp_loss(const double* d_part, int nb, int64_t B, cudaStream_t s) {
@@ -416,51 +413,54 @@ static double mlp_loss(const double* d_part, int nb, int64_t B, cudaStream_t s) 
   return loss / double(B);
 }
 
+// gradients from a.dY on
+static void backward64(const double* P, const double* X, int64_t B, MlpActs<double>& a, double* G,
+                       cudaStream_t s) {
+  MlpOffsets o;
+  const int64_t np = mlp_n_params();
+  const int64_t nh = B * kWd;
+  // output layer
+  gemm(G + o.w4, kWd, a.dY.p, 1, true, a.H3.p, kWd, false, 1, kWd, int(B), B, nh, np - o.w4, s);
+  k_colsum<<<1, 32, 0, s>>>(a.dY.p, B, 1, G + o.b4);
+  DMRG_LAUNCHED();
+  gemm(a.dH.p, kWd, a.dY.p, 1, false, P + o.w4, kWd, false, int(B), kWd, 1, B, np - o.w4, nh, s);
+  // layer 3
+  k_relu_grad<<<grid_for(nh), 256, 0, s>>>(a.Z3.p, a.dH.p, nh);
+  DMRG_LAUNCHED();
+  gemm(G + o.W3, kWd, a.dH.p, kWd, true, a.H2.p, kWd, false, kWd, kWd, int(B), nh, nh,
+          np - o.W3, s);
+  k_colsum<<<1, kWd, 0, s>>>(a.dH.p, B, kWd, G + o.b3);
+  DMRG_LAUNCHED();
+  gemm(a.dZ.p, kWd, a.dH.p, kWd, false, P + o.W3, kWd, false, int(B), kWd, kWd, nh, np - o.W3,
+          nh, s);
+  // layer 2
+  k_relu_grad<<<grid_for(nh), 256, 0, s>>>(a.Z2.p, a.dZ.p, nh);
+  DMRG_LAUNCHED();
+  gemm(G + o.W2, kWd, a.dZ.p, kWd, true, a.H1.p, kWd, false, kWd, kWd, int(B), nh, nh,
+          np - o.W2, s);
+  k_colsum<<<1, kWd, 0, s>>>(a.dZ.p, B, kWd, G + o.b2);
+  DMRG_LAUNCHED();
+  gemm(a.dH.p, kWd, a.dZ.p, kWd, false, P + o.W2, kWd, false, int(B), kWd, kWd, nh, np - o.W2,
+          nh, s);
+  // layer 1
+  k_relu_grad<<<grid_for(nh), 256, 0, s>>>(a.Z1.p, a.dH.p, nh);
+  DMRG_LAUNCHED();
+  gemm(G + o.W1, kIn, a.dH.p, kWd, true, X, kIn, false, kWd, kIn, int(B), nh, B * kIn,
+          np - o.W1, s);
+  k_colsum<<<1, kWd, 0, s>>>(a.dH.p, B, kWd, G + o.b1);
+  DMRG_LAUNCHED();
+}
+
 // loss (mean squared error) and gradient G of the parameters; forward must have run on X
 template <class T>
 double mlp_backward(const T* P, const T* X, const T* Tg, int64_t B, MlpActs<T>& a, T* G,
                     cudaStream_t s) {
-  MlpOffsets<T> o;
-  const int64_t np = mlp_n_params();
-  const int64_t nh = B * kWd;
   const int nb = 64;
   a.part.alloc(nb);
   k_mse<T><<<nb, 256, 0, s>>>(a.Y.p, Tg, B, a.dY.p, a.part.p);
   DMRG_LAUNCHED();
-  if constexpr (std::is_same<T, float>::value) {
-    backward32(P, X, B, a, G, s);
-    return mlp_loss(a.part.p, nb, B, s);
-  }
-  // output layer
-  gemm<T>(G + o.w4, kWd, a.dY.p, 1, true, a.H3.p, kWd, false, 1, kWd, int(B), B, nh, np - o.w4, s);
-  k_colsum<T><<<1, 32, 0, s>>>(a.dY.p, B, 1, G + o.b4);
-  DMRG_LAUNCHED();
-  gemm<T>(a.dH.p, kWd, a.dY.p, 1, false, P + o.w4, kWd, false, int(B), kWd, 1, B, np - o.w4, nh, s);
-  // layer 3
-  k_relu_grad<T><<<grid_for(nh), 256, 0, s>>>(a.Z3.p, a.dH.p, nh);
-  DMRG_LAUNCHED();
-  gemm<T>(G + o.W3, kWd, a.dH.p, kWd, true, a.H2.p, kWd, false, kWd, kWd, int(B), nh, nh,
-          np - o.W3, s);
-  k_colsum<T><<<1, kWd, 0, s>>>(a.dH.p, B, kWd, G + o.b3);
-  DMRG_LAUNCHED();
-  gemm<T>(a.dZ.p, kWd, a.dH.p, kWd, false, P + o.W3, kWd, false, int(B), kWd, kWd, nh, np - o.W3,
-          nh, s);
-  // layer 2
-  k_relu_grad<T><<<grid_for(nh), 256, 0, s>>>(a.Z2.p, a.dZ.p, nh);
-  DMRG_LAUNCHED();
-  gemm<T>(G + o.W2, kWd, a.dZ.p, kWd, true, a.H1.p, kWd, false, kWd, kWd, int(B), nh, nh,
-          np - o.W2, s);
-  k_colsum<T><<<1, kWd, 0, s>>>(a.dZ.p, B, kWd, G + o.b2);
-  DMRG_LAUNCHED();
-  gemm<T>(a.dH.p, kWd, a.dZ.p, kWd, false, P + o.W2, kWd, false, int(B), kWd, kWd, nh, np - o.W2,
-          nh, s);
-  // layer 1
-  k_relu_grad<T><<<grid_for(nh), 256, 0, s>>>(a.Z1.p, a.dH.p, nh);
-  DMRG_LAUNCHED();
-  gemm<T>(G + o.W1, kIn, a.dH.p, kWd, true, X, kIn, false, kWd, kIn, int(B), nh, B * kIn,
-          np - o.W1, s);
-  k_colsum<T><<<1, kWd, 0, s>>>(a.dH.p, B, kWd, G + o.b1);
-  DMRG_LAUNCHED();
+  if constexpr (std::is_same<T, float>::value) backward32(P, X, B, a, G, s);
+  else backward64(P, X, B, a, G, s);
   return mlp_loss(a.part.p, nb, B, s);
 }
 
