@@ -16,8 +16,9 @@
 // shared-memory buffer while this one is multiplied (terms up to 32 wide whole, 16 bytes a copy;
 // of wider ones a 32 x 32 part, rows of 36 words).  32 KB per unit, so seven units (28 warps) on
 // an SM, against twelve warps with a ring of terms per warp; terms wider than 32 are pipelined
-// like the others instead of staged and waited for.  The kernel is bound by instruction issue
-// (74 % of the slots), so the copies and the bounds are what is kept short.
+// like the others instead of staged and waited for.  On starting-state blocks the first version, with
+// 4-byte copies, was bound by instruction issue (74 % of the slots), so the copies and the bounds are
+// what is kept short; on small terms the kernel now waits for their loads (37 % of the slots).
 //   The high part is rounded with integer operations (add half a unit, cut): the conversion
 // instruction runs at a quarter of their rate and was half of the inner loop's time with two per
 // operand element.  The low part keeps it, so that a NaN stays one.
@@ -156,8 +157,8 @@ __device__ __forceinline__ Mine my_tiles(int MT, int NT, int warp) {
   return w;
 }
 
-// W = 4 warps for tiles of up to 32 columns, 2 for narrow ones (half of the warps would have no
-// MMA tile there)
+// W = 4 warps for tiles of up to 32 columns, 2 for narrow ones when they have a launch of their own
+// (half of the warps would have no MMA tile there)
 template <int W>
 __global__ void __launch_bounds__(32 * W, W == 4 ? 7 : 8)
 k_heff_tc(const HeffTile* __restrict__ tiles, const int32_t* __restrict__ order,

@@ -1,5 +1,5 @@
-// Device functions of the FP64 symmetric eigensolver shared by the density-matrix and the Ritz
-// kernels.
+// Device functions of the FP64 symmetric eigensolver of the density-matrix kernels (kernels.cu).  The
+// Ritz problem of Davidson has its own, with the same pairing and rotations (davidson.cu).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
