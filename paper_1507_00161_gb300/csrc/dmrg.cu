@@ -1022,8 +1022,16 @@ static OpSet vacuum_ops(int nlab, int which, cudaStream_t s) {
   return v;
 }
 
-// Whether the mixed kernels of a product run side by side (tile_kernels), the wide and the narrow tiles
-// as launches of their own; otherwise one after the other, with one launch for all tiles.  Two
+// Whether the kernels of an FP64 product run side by side (tile_kernels): small blocks, tiles and grouped
+// passes, two of which have work.  Measured (GB300), one stream against two: pf 8p+8n at position 5 353
+// -> 229 us, sd 4p+4n at position 4 (two tiles) 153 -> 140; without grouped passes pf 4p+4n at position 9,
+// M0 = 256, 6 us of 280 per product of a Davidson run, the smallest product 39 -> 38 us.
+static bool two_kernels(int64_t n_stiles, int64_t n_tiles, bool any_big) {
+  return (n_stiles > 0) + (n_tiles > 0) + any_big >= 2;
+}
+
+// The same for the mixed kernels, and whether the wide and the narrow tiles are launches of their
+// own; otherwise they run one after the other, with one launch for all tiles.  Two
 // streams cost host calls in an eager product and 10 to 40 us in the capture at the second one, which
 // every new superblock pays.  Beside grouped passes a few tiles repay that: measured (GB300; repeated
 // product, second product), pf 4p+4n at position 4 (18 tiles) 213 -> 198 us and 314 -> 325, pf 8p+8n at
@@ -1317,7 +1325,9 @@ static void build_super(Ctx& c, int p) {
     std::vector<int32_t> order;
     const bool any_big = std::find(big_bo.begin(), big_bo.end(), 1) != big_bo.end();
     sb->beside = tiles_beside(int64_t(tl.size()), any_big);
-    if (sb->beside || (any_big && !tl.empty())) c.side.create();   // (70 us: not in the first product)
+    const bool two = two_kernels(int64_t(tls.size()), int64_t(tl.size()), any_big);
+    if (c.opt.precision == DMRG_FP64 ? two : sb->beside)
+      c.side.create();   // (70 us: not in the first product)
     sb->n_fwide = heff_tc_order(tl, sb->beside, order);
     sb->forder.upload(order, c.stream);
     sb->stiles.upload(tls, c.stream);
@@ -1551,12 +1561,10 @@ struct TileLists {
 template <class F>
 static void tile_kernels(const TileLists& l, const HeffPtrs<double>& p, SideStream& side,
                          cudaStream_t st, bool any_big, F&& big) {
-  // the tiles beside the grouped passes (few long chains each): pf 8p+8n at position 5 353 -> 229 us,
-  // sd 4p+4n at position 4 (two tiles) 153 -> 140; the small blocks alone are not worth a second stream
-  const bool fork = any_big && l.n_tiles > 0;
+  const bool fork = two_kernels(l.n_stiles, l.n_tiles, any_big);
   cudaStream_t sd = fork ? side.begin(st) : st;
   heff_small<double>(l.stiles, l.n_stiles, l.items, p, sd);
-  heff_fused64(l.tiles, l.n_tiles, l.items, p, sd);
+  heff_fused64(l.tiles, l.n_tiles, l.items, p, any_big ? sd : st);
   if (any_big) big();
   if (fork) side.end(st);
   heff_reduce_slots<double>(l.red, l.n_plain, l.n_red, p, st);
