@@ -24,7 +24,7 @@
 // formed by different warps.
 //
 // Measured (GB300), chain and Ritz problem together, against 15 launches and two readbacks per
-// iteration, bit for bit the same results: with the products' changes a Davidson run of pf 4p+4n
+// iteration, the same results to the bit in every run compared: with the products' changes a Davidson run of pf 4p+4n
 // (n = 700, ~55 products) 45.9 -> 19.2 ms, an sd-shell sweep at M = 64 200 -> 120 ms, five instances
 // in batch mode 505 -> 316 ms; residual and first orthogonalisation at n = 300 13.7 + 11.5 -> 9.3 + 7.8 us.
 #include <math.h>
